@@ -38,6 +38,7 @@ int op_project_scalar(const cffyn_shell*, const double*, double*, cudaStream_t, 
 int op_project(const cffyn_shell*, const double*, double*, const int*, int, const int* const[3],
                const int[3], cudaStream_t, int);
 int op_prepare(const cffyn_shell*, const double*, bool, int, long long, int, cudaStream_t);
+bool op_dft_persistent(const cffyn_shell*, int);
 // setup.cu
 int build_operators(cffyn_shell*);
 int build_tc_family(cffyn_shell*, int);
@@ -271,6 +272,7 @@ static int create_shell(const cffyn_shell_desc* desc, int ns, cffyn_shell** out)
   sh->nC[0] = 11 + sh->ng;
   sh->P = (size_t)d.n_r * d.n_theta * d.n_phi;
   cudaGetDevice(&sh->device);
+  cudaDeviceGetAttribute(&sh->sm_count, cudaDevAttrMultiProcessorCount, sh->device);
   {
     const double pi = 3.14159265358979323846;
     double r0 = 0.5 * (d.r_out + d.r_in) - 0.5 * (d.r_out - d.r_in);
@@ -540,8 +542,8 @@ static const double* stage_state_of(const cffyn_shell* sh, const double* u, int 
 // 16 real spin-0 slots and the first 4 spin-1 pairs) and the rest (the other
 // spin-1 pairs, spin 2, spin 3 and the gauge slots).  Each half is a whole
 // set of projection classes, so the chains share no buffer; each fills the
-// partly empty last wave of the other's launches (3.228 -> 3.135 ms per step
-// on the 33 x 48 x 96 shell).
+// SMs that the other's small launches leave idle.  Where a half's launches run
+// on the persistent kernel, which fills the device alone, one chain is used.
 constexpr int kSplitR0 = 16, kSplitC1 = 4, kSplitSlots = kSplitR0 + 2 * kSplitC1;
 
 // filter of the functions in `spin` (in place through D and D + nvP): the
@@ -561,7 +563,7 @@ static int filter_in_step(cffyn_shell* sh, double* spin, cudaStream_t st, Run&& 
   if ((r = run(10, [&] { return op_prepare(sh, spin, true, nf, (long long)sh->P, pairing, st); })))
     return r;
   if (conc && yn && sh->d.precision == CFFYN_MIXED && sh->aux_stream && sh->nR0 >= kSplitR0 &&
-      sh->nC[0] >= kSplitC1) {
+      sh->nC[0] >= kSplitC1 && !op_dft_persistent(sh, kSplitSlots * sh->ns)) {
     cudaStream_t sa = sh->aux_stream;
     const int fa = kSplitSlots * sh->ns;  // arrays of the first half (stacked: [slot][shell])
     const int* ca[3] = {cl[0], nullptr, nullptr};

@@ -71,6 +71,7 @@ struct cffyn_shell {
   double dt_default;
   size_t bytes = 0;
   int device = 0;
+  int sm_count = 1;             // SMs of the device: CTAs of a persistent launch
 
   // grid (device)
   double *r = nullptr, *sth = nullptr, *cth = nullptr, *sph = nullptr, *cph = nullptr;

@@ -67,6 +67,9 @@ struct OpArgs {
   int fld0;              // OP_ROWS: array index of the launch's first array (its exponent word, pairing)
 };
 
+// Column c of a launch, with 32-bit divisions: a column has at least three
+// values and the workspace holds seven or eight arrays of them, so c < 2^31
+// on any device that can hold the shell.
 __device__ __forceinline__ ColDesc make_col(const OpArgs& a, long long c) {
   ColDesc d;
   d.valid = c < a.g.ncols;
@@ -74,14 +77,14 @@ __device__ __forceinline__ ColDesc make_col(const OpArgs& a, long long c) {
   if (!d.valid) c = 0;
   switch (a.kind) {
     case OP_R: {
-      d.fld = (int)(c / ((long long)a.J * a.N));
+      d.fld = (int)((unsigned)c / (unsigned)(a.J * a.N));
       d.in0 = c * a.n_r;
       d.out0 = d.in0;
       d.in1 = d.out1 = 0;
       break;
     }
     case OP_ROWS: {
-      long long b = c / a.Q, q = c - b * a.Q;
+      const long long b = (unsigned)c / (unsigned)a.Q, q = c - b * a.Q;
       d.fld = a.fld0 + (int)b;
       d.in0 = b * a.in_bs + q;
       d.out0 = b * a.out_bs + q;
@@ -89,10 +92,10 @@ __device__ __forceinline__ ColDesc make_col(const OpArgs& a, long long c) {
       break;
     }
     case OP_THETA: {
-      long long pb = c / a.n_r;
+      const long long pb = (unsigned)c / (unsigned)a.n_r;
       int kr = (int)(c - pb * a.n_r);
       int half = a.J / 2;
-      long long mu = pb / half;
+      const long long mu = (unsigned)pb / (unsigned)half;
       int jp = (int)(pb - mu * half);
       d.fld = (int)mu;
       d.in0 = ((mu * a.J + jp) * a.N) * a.n_r + kr;
@@ -107,10 +110,10 @@ __device__ __forceinline__ ColDesc make_col(const OpArgs& a, long long c) {
       int nparts = a.m == 0 ? 1 : 2;
       long long per = (long long)nparts * a.n_r;
       if (c >= per * a.nslots * a.ns) { d.valid = 0; c = 0; }
-      long long fi = c / per;
+      const long long fi = (unsigned)c / (unsigned)per;
       int rem = (int)(c - fi * per);
       int part = rem / a.n_r, kr = rem - part * a.n_r;
-      const long long fs = fi / a.ns;
+      const long long fs = (unsigned)fi / (unsigned)a.ns;
       int f = a.slots[fs < a.nslots ? fs : 0] * a.ns + (int)(fi - fs * a.ns);
       d.fld = f;
       int row = part == 0 ? a.m : a.L + a.m;
@@ -125,10 +128,10 @@ __device__ __forceinline__ ColDesc make_col(const OpArgs& a, long long c) {
       int nparts = a.m == 0 ? 2 : 4;
       long long per = (long long)nparts * a.n_r;
       if (c >= per * a.nslots * a.ns) { d.valid = 0; c = 0; }
-      long long pi = c / per;
+      const long long pi = (unsigned)c / (unsigned)per;
       int rem = (int)(c - pi * per);
       int part = rem / a.n_r, kr = rem - part * a.n_r;
-      const long long ps = pi / a.ns;
+      const long long ps = (unsigned)pi / (unsigned)a.ns;
       int fre = a.slots[ps < a.nslots ? ps : 0] * a.ns + (int)(pi - ps * a.ns), fim = fre + a.ns;
       d.fld = fre;
       int ra = a.m, rb = a.L + a.m;
@@ -159,20 +162,6 @@ __device__ __forceinline__ double load_elem(const OpArgs& a, const ColDesc& d, i
   const double v = __ldg(a.in + d.in1 + (long long)kk * a.g.in_rs);
   // sign flip on the bit pattern (no FP64 instruction)
   return __longlong_as_double(__double_as_longlong(v) ^ ((long long)d.sgn1 << 63));
-}
-
-// Raw 64-bit element of a column for the split-precision core: an FP64 word
-// (FI = false) or a (hi, lo) float pair (FI = true), sign applied on the bits.
-template <bool FI>
-__device__ __forceinline__ long long load_raw(const OpArgs& a, const ColDesc& d, int k) {
-  if (!d.valid || k >= a.g.K) return 0;
-  const long long* in = reinterpret_cast<const long long*>(a.in);
-  if (k < a.g.K0) return __ldg(in + d.in0 + (long long)k * a.g.in_rs);
-  if (d.sgn1 == 2) return 0;
-  int kk = a.g.rev1 ? (a.g.K - 1 - k) : (k - a.g.K0);
-  const long long w = __ldg(in + d.in1 + (long long)kk * a.g.in_rs);
-  const long long m = FI ? (long long)0x8000000080000000ull : (long long)0x8000000000000000ull;
-  return d.sgn1 ? (w ^ m) : w;
 }
 
 __device__ __forceinline__ void store_elem(const OpArgs& a, const ColDesc& d, int p, double v) {
@@ -408,26 +397,34 @@ __global__ void __launch_bounds__(kExpThreads) k_field_exp(const long long* __re
 // ---------------------------------------------------------------------------
 // Split-precision core on the fifth-generation tensor cores (tcgen05).
 //
-// CTA: 128 data columns (the MMA's M: one TMEM lane each) x one row group of
-// W (N = 48 or 96 rows), all of K in k-steps of 16 through a ring of
-// shared-memory stages.  Warp-specialised:
-//   producer warps (256 or 512 threads; one column and KQ = 8 or 4
-//     consecutive k of every k-step each): write the six BF16 digit slices of
-//     their values (47-bit fixed point relative to the field's exponent; the
-//     next k-step's input words loaded right after the arrive) into the
-//     stage, then arrive on its `xfull` barrier; after the last k-step they
-//     run the epilogue;
-//   one MMA warp: bulk-copies (TMA) the operator's sixteen slices of each
-//     k-step (see TcOp) a stage ahead and, once a stage is full, issues the
-//     digit-pair MMAs into five FP32 accumulators in TMEM and commits them to
-//     the stage's `empty` barrier:
+// Work item: 128 data columns (the MMA's M: one TMEM lane each) x one row
+// group of W (ROWS = 48 or 96 rows), all of K in k-steps of 16.  A launch is
+// persistent: one CTA per SM takes items blockIdx.x, + gridDim.x, ... of all
+// its operator classes and azimuthal numbers.  Warp-specialised, every role
+// walking the same item list on its own:
+//   producer warps (three groups of 128 threads; a thread has one column and
+//     all 16 k of every third k-step): load the raw words, cut them into six
+//     BF16 digit slices (47-bit fixed point relative to the field's exponent)
+//     in a shared-memory stage, arrive on its `xfull`; the loads of the
+//     group's next k-step are issued right after the arrive (the proxy fence
+//     and the arrive's release wait for every load the thread has in flight);
+//   loader warp: bulk-copies (TMA) the operator's slices of each k-step (see
+//     TcOp) into the stage, completing on its `wfull`;
+//   MMA warp: once a stage is full, issues the digit-pair MMAs into five FP32
+//     accumulators in TMEM and commits them to the stage's `empty`; after an
+//     item's last k-step commits `accfull`;
+//   epilogue warps (two per 32 TMEM lanes, half the rows each): read the
+//     accumulators, fold them into float pairs, store, release `accempty`.
+// The ring of stages runs across items, so the loads, the slicing and the
+// operator copies of the next items go on under the products and the
+// epilogue of the current one; with 48 rows the accumulators are
+// double-buffered too (2 x 240 of the 512 TMEM columns), with 96 rows (480
+// columns) the products wait for the fold's last TMEM load.
 //   acc_d = sum_{i+j=d} W_i X_j                            d = 0..3
 //   acc_4 = sum_{i+j=4} W_i X_j + 2^-8 sum_{i+j=5} W_i X_j + 2^-16 sum_{i+j=6} W_i X_j
 // The digit-sum <= 4 pairs of one input slice X_j go out as one MMA of up to
 // 256 rows over adjacent operator slices into adjacent accumulators (fewer
 // MMAs per k-step, each input slice read from shared memory fewer times).
-// A block's time goes mostly to the producers' loads and slicing, to its
-// set-up and to the epilogue; the tensor core is busy about a third of it.
 // The digit-sum-6 pairs are issued for the derivatives only (TcBatch::sum6);
 // the filter's DFTs and projections stop at digit sum 5 (21 pairs) and copy
 // eleven operator slices per k-step.
@@ -438,7 +435,7 @@ __global__ void __launch_bounds__(kExpThreads) k_field_exp(const long long* __re
 // result is as accurate as the 47-bit fixed point of its inputs; without
 // them the dropped digit-sum-6 products (weight 2^-48) were the largest
 // error.  The epilogue sums (acc_0 + acc_1 2^-8 + ... + acc_4 2^-32)
-// 2^(E_row + E_col - 14) as a float pair (fold_pair).
+// 2^(E_row + E_col - 14) as a float pair (fold_pairs).
 
 constexpr int kTcCols = 128;
 constexpr int kTcXSlice = kTcCols * 16 * 2;                 // bytes of one data slice per k-step
@@ -452,18 +449,529 @@ __device__ __forceinline__ bool pipe_wait(uint64_t* b, unsigned parity, unsigned
 }
 
 // Up to four operator applications with the same row-group size in one
-// launch (the projections of the spin classes); blockIdx.y = class * nm + m.
+// launch (the projections of the spin classes).
 constexpr int kMaxBatch = 4;
 struct TcBatch {
   OpArgs a[kMaxBatch];
   TcOp W[kMaxBatch];
-  long long tiles[kMaxBatch];  // column tiles of each class
+  int tiles[kMaxBatch];      // column tiles of each class (per azimuthal number)
+  int first[kMaxBatch + 1];  // first work item of each class; the number of items
   int nclass, nm;
   int eoff;  // added to every column exponent: a bound from an earlier scan times the operator gain
   int sum6;  // issue the digit-sum-6 pairs (derivatives); the filter's operators stop at digit sum 5
   unsigned long long wait_ns;  // bound of every pipeline wait (the shell's setting; 0: give up at once)
 };
 
+// thread layout of a CTA
+constexpr int kEpiWarps = 8, kProdGroups = 3;
+constexpr int kProdWarp0 = kEpiWarps, kMmaWarp = kProdWarp0 + 4 * kProdGroups, kLoadWarp = kMmaWarp + 1;
+constexpr int kWsThreads = 32 * (kLoadWarp + 1);  // 704
+
+template <int ROWS>
+struct WsCfg {
+  static constexpr int kWSlice = ROWS * 16 * 2;                        // bytes of one operator slice
+  static constexpr int kWBytes = kTcWSlices * kWSlice;                 // 24576 | 49152
+  static constexpr int kStage = kTcXBytes + kWBytes;                   // 49152 | 73728
+  static constexpr int kAccs = ROWS == 48 ? 2 : 1;                     // accumulator sets in TMEM
+  static constexpr uint32_t kTmemCols = 512;                           // set i at column 256 i
+  static_assert(kStage % 1024 == 0, "stage alignment of the descriptors and bulk copies");
+};
+// stages of the ring; the staged epilogue of d_r takes one stage's room for
+// the outputs (see stage_bytes)
+template <int ROWS, bool STAGE>
+constexpr int kRingStages = (ROWS == 48 ? 4 : 3) - (STAGE ? 1 : 0);
+constexpr int kTcMaxSmem = 224 * 1024;  // of 227 KB, beside the barriers and row factors
+
+// One work item: class, azimuthal number, column tile, row group.
+struct TcItem {
+  int cls, m, grp, ksteps;
+  long long tile;
+};
+
+__device__ __forceinline__ TcItem item_at(const TcBatch& B, int t) {
+  TcItem x;
+  x.cls = 0;
+#pragma unroll
+  for (int c = 1; c < kMaxBatch; ++c)
+    if (c < B.nclass && t >= B.first[c]) x.cls = c;
+  const int ng = B.W[x.cls].ngroups;
+  unsigned q = (unsigned)(t - B.first[x.cls]);
+  x.grp = ng == 1 ? 0 : (int)(q % (unsigned)ng);
+  q = ng == 1 ? q : q / (unsigned)ng;
+  x.m = B.a[x.cls].batched_m ? (int)(q / (unsigned)B.tiles[x.cls]) : 0;
+  x.tile = (long long)(q - (unsigned)x.m * (unsigned)B.tiles[x.cls]);
+  x.ksteps = B.W[x.cls].ksteps;
+  return x;
+}
+
+// Packed FP32 pairs (both halves rounded to nearest, never contracted).
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_dup(float a) { return f2_pack(a, a); }
+__device__ __forceinline__ unsigned int f2_lo(f2 a) { return (unsigned int)a; }
+__device__ __forceinline__ unsigned int f2_hi(f2 a) { return (unsigned int)(a >> 32); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// Raw 64-bit words of 16 consecutive k of one column (zero outside K or in an
+// empty second segment; the sign of a negated segment applied on the bits).
+// A run inside one segment takes one pointer and its stride (an invalid
+// column reads column 0, whose results are not stored); only a run that
+// crosses segments or the end of K checks every element.  Branch-free within
+// a run so that the loads issue together.
+template <bool FI>
+__device__ __forceinline__ void gather16(const OpArgs& a, const ColDesc& d, int k0, long long (&w)[16]) {
+  const long long* in = reinterpret_cast<const long long*>(a.in);
+  const long long m = FI ? (long long)0x8000000080000000ull : (long long)0x8000000000000000ull;
+  const int K = a.g.K, K0 = a.g.K0;
+  // element k of segment s lives at q_s[k * rs_s]
+  const int rs0 = a.g.in_rs, rs1 = a.g.rev1 ? -rs0 : rs0;
+  const long long* q0 = in + d.in0;
+  const long long* q1 = in + d.in1 + (a.g.rev1 ? (K - 1) * rs0 : -(K0 * rs0));
+  const bool flip = d.sgn1 == 1;
+  const int kend = d.sgn1 == 2 ? min(K, K0) : K;
+  const bool s0 = k0 + 16 <= min(kend, K0), s1 = k0 >= K0 && k0 + 16 <= kend;
+  if (__all_sync(0xffffffffu, s0 || s1)) {
+    const long long step = s1 ? rs1 : rs0;
+    const long long* p = (s1 ? q1 : q0) + k0 * step;
+#pragma unroll
+    for (int i = 0; i < 16; ++i, p += step) w[i] = __ldg(p);
+    if (s1 && flip) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) w[i] ^= m;
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int k = k0 + i;
+    const bool seg1 = k >= K0;
+    const long long* p = seg1 ? q1 + k * rs1 : q0 + k * rs0;
+    const long long v = k < kend ? __ldg(p) : 0ll;
+    w[i] = seg1 && flip ? (v ^ m) : v;
+  }
+}
+
+// 2^k as a float, k clamped to the normal range
+__device__ __forceinline__ float pow2f(int k) {
+  return __int_as_float((max(-126, min(127, k)) + 127) << 23);
+}
+
+// a + b c (c a power of two), rounded, and its error, exactly (TwoSum with the
+// product inside the fused additions: b c is exact).
+__device__ __forceinline__ void f2_two_sum_scaled(f2 a, f2 b, f2 c, f2& s, f2& e) {
+  s = f2_fma(b, c, a);
+  const f2 nb = f2_sub(a, s);
+  e = f2_add(f2_sub(a, f2_add(s, nb)), f2_fma(b, c, nb));
+}
+
+// (hi, lo) float pairs of rows j and j + 1, packed like the mixed path's
+// internal storage, of (a0 + a1 2^-8 + a2 2^-16 + a3 2^-24 + a4 2^-32) f (f powers
+// of two; the halves of every operand are the two rows).
+// a0 + a1 2^-8 + a2 2^-16 + a3 2^-24 (exact values) is summed with error-free
+// transformations, so that the sum's only roundings are those of the low
+// words and of a4 2^-32 (below 2^-48 of |a0|); summing a3 2^-24 in plain FP32
+// would cost about 2^-24 of it, more than the digit-sum-6 terms.  Packed FP32
+// arithmetic: the FMA pipe takes as long as for two scalar folds, but half
+// the issue slots, which the producers share.
+__device__ __forceinline__ void fold_pairs(f2 a0, f2 a1, f2 a2, f2 a3, f2 a4, f2 f, f2& hi, f2& lo) {
+  f2 s, t, e0, e1, e2;
+  f2_two_sum_scaled(a0, a1, f2_dup(0.00390625f), s, e0);
+  f2_two_sum_scaled(s, a2, f2_dup(1.52587890625e-05f), t, e1);
+  f2_two_sum_scaled(t, a3, f2_dup(5.9604644775390625e-08f), s, e2);
+  const f2 low = f2_fma(a4, f2_dup(2.3283064365386963e-10f), f2_add(f2_add(e0, e1), e2));
+  hi = f2_add(s, low);
+  lo = f2_mul(f2_sub(low, f2_sub(hi, s)), f);
+  hi = f2_mul(hi, f);
+}
+
+// The outputs of a column scale by 2^E_row 2^ec, in one product of the two;
+// where ec is extreme that product can leave the float range, and the factors
+// (2^ec in two parts, the second beyond the float range's) go one by one.
+struct ColScale {
+  f2 f1, f2_;
+  bool extreme;
+  __device__ __forceinline__ explicit ColScale(int ec)
+      : f1(f2_dup(pow2f(ec))), f2_(f2_dup(pow2f(ec - max(-126, min(127, ec))))), extreme(ec < -60 || ec > 60) {}
+};
+
+// The folded pairs of rows j and j + 1 of a chunk of accumulator rows v;
+// rowF: those rows' 2^E_row (8-byte aligned).
+template <int N>
+__device__ __forceinline__ void fold_rows(const uint32_t (&v)[5][N], int j, const float* rowF, const ColScale& cs,
+                                          long long& w0, long long& w1) {
+  auto two = [&](int d) { return f2_pack(__uint_as_float(v[d][j]), __uint_as_float(v[d][j + 1])); };
+  const float2 rr = *reinterpret_cast<const float2*>(rowF);
+  const f2 rf = f2_pack(rr.x, rr.y);
+  f2 hi, lo;
+  fold_pairs(two(0), two(1), two(2), two(3), two(4), cs.extreme ? rf : f2_mul(rf, cs.f1), hi, lo);
+  if (cs.extreme) {
+    hi = f2_mul(f2_mul(hi, cs.f1), cs.f2_);
+    lo = f2_mul(f2_mul(lo, cs.f1), cs.f2_);
+  }
+  w0 = (long long)((lo << 32) | f2_lo(hi));
+  w1 = (long long)((lo & 0xffffffff00000000ull) | f2_hi(hi));
+}
+
+// Digit slices of two float pairs x = hi + lo (|lo| < ulp(hi), |x| < 2^E) on
+// the FMA pipe, packed.  Digit j has weight 2^(E - 7 - 8j) (the balanced
+// base-256 digits of round(x 2^(47 - E))).  With v = x 2^(7 - E) (sc, exact)
+// and s = -(remainder), the exact steps
+//   d_0 = rint(v), s = d_0 - v;   d_j = rint(-256 s), s = d_j + 256 s
+// (rint by adding and subtracting 1.5 * 2^23) give balanced digits |d| <= 128
+// of hi; the last digit rounds like the fixed-point conversion.  lo
+// contributes to digits 3..5 only (|lo| / w_2 < 1/2; sc3 = sc 2^24), so digit
+// j is d_j(hi) + d_j(lo), |.| <= 256, an exact BF16 value; it is the same
+// integer sum of weights as the rounded fixed point of hi plus that of lo.
+// Requires -78 <= E <= 126 (every weight and inverse weight a normal float).
+// out[j]: the two values' digits as BF16 (the upper half of the float).
+__device__ __forceinline__ void digits_two(long long x0, long long x1, f2 sc, f2 sc3, unsigned int (&out)[kSlices]) {
+  const f2 M = f2_dup(12582912.0f), up = f2_dup(256.0f), dn = f2_dup(-256.0f);  // 1.5 * 2^23
+  const f2 v = f2_mul(f2_pack(__int_as_float((int)(unsigned int)x0), __int_as_float((int)(unsigned int)x1)), sc);
+  const f2 u = f2_mul(f2_pack(__int_as_float((int)(unsigned int)((unsigned long long)x0 >> 32)),
+                              __int_as_float((int)(unsigned int)((unsigned long long)x1 >> 32))),
+                      sc3);
+  f2 d[kSlices];
+  d[0] = f2_sub(f2_add(v, M), M);
+  f2 s = f2_sub(d[0], v);
+#pragma unroll
+  for (int j = 1; j < kSlices; ++j) {
+    d[j] = f2_sub(f2_fma(s, dn, M), M);
+    if (j < kSlices - 1) s = f2_fma(s, up, d[j]);
+  }
+  f2 e = f2_sub(f2_add(u, M), M);
+  s = f2_sub(e, u);
+  d[3] = f2_add(d[3], e);
+#pragma unroll
+  for (int j = 4; j < kSlices; ++j) {
+    e = f2_sub(f2_fma(s, dn, M), M);
+    if (j < kSlices - 1) s = f2_fma(s, up, e);
+    d[j] = f2_add(d[j], e);
+  }
+#pragma unroll
+  for (int j = 0; j < kSlices; ++j) out[j] = __byte_perm(f2_lo(d[j]), f2_hi(d[j]), 0x7632);
+}
+
+__device__ __forceinline__ void bar_arrive(uint64_t* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(b)) : "memory");
+}
+// named barrier over nthreads threads, and the AND of their predicates
+__device__ __forceinline__ void named_sync(int id, int nthreads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+__device__ __forceinline__ bool named_and(int id, int nthreads, bool p) {
+  int r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.s32 p, %3, 0;\nbar.red.and.pred q, %1, %2, p;\nselp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(id), "r"(nthreads), "r"((int)p)
+      : "memory");
+  return r != 0;
+}
+
+// exponent of a column's fixed point, relative to 1022 in the field words
+__device__ __forceinline__ int col_exponent(const TcBatch& B, const OpArgs& a, const ColDesc& col,
+                                            const int* __restrict__ exps, int pairing) {
+  int ce = exps[col.fld];
+  if (pairing) {
+    // slot pairs (f, f ^ 1), f >= kPairedFrom, of the same stacked shell
+    const int f = a.ns == 1 ? col.fld : col.fld / a.ns, sidx = col.fld - f * a.ns;
+    if (f >= kPairedFrom) ce = max(ce, exps[(f ^ 1) * a.ns + sidx]);
+  }
+  return ce - 1022 + B.eoff;
+}
+
+// STAGE: the launch is d_r (one operator class, all rows in one group): the
+// epilogue stages a tile's outputs in shared memory and stores them as one
+// contiguous block per 32 columns.
+template <bool FI, int ROWS, bool STAGE = false>
+__global__ void __launch_bounds__(kWsThreads, 1)
+    k_op_ws(const __grid_constant__ TcBatch B, const int* __restrict__ exps, int pairing, int* __restrict__ flag) {
+  using C = WsCfg<ROWS>;
+  constexpr int S = kRingStages<ROWS, STAGE>, A = C::kAccs;
+  extern __shared__ __align__(1024) unsigned char smtc[];
+  __shared__ uint64_t xfull[S], wfull[S], empty[S], accfull[A], accempty[A], drained;
+  __shared__ uint32_t tmem_base;
+  __shared__ __align__(16) float rowF[kEpiWarps][ROWS / 2];  // 2^E_row of each epilogue warp's rows
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int total = B.first[B.nclass];
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      tc::bar_init(&xfull[s], 128);
+      tc::bar_init(&wfull[s], 1);
+      tc::bar_init(&empty[s], 1);
+    }
+    for (int i = 0; i < A; ++i) {
+      tc::bar_init(&accfull[i], 1);
+      tc::bar_init(&accempty[i], kEpiWarps);
+    }
+    tc::bar_init(&drained, 1);
+  }
+  if (warp == kMmaWarp) tc::alloc(&tmem_base, C::kTmemCols);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tm = tmem_base;
+  bool ok = true;
+
+  if (warp >= kProdWarp0 && warp < kMmaWarp) {
+    // a group must not be two uses of a stage ahead of the products (its wait
+    // on `empty` tells phases apart by their parity only): with two stages
+    // the third group has no part
+    constexpr int G = S < kProdGroups ? S : kProdGroups;
+    const int g = (warp - kProdWarp0) >> 2;
+    const int ctile = (warp & 3) * 32 + lane;
+    const int xoff = (ctile >> 3) * 256 + (ctile & 7) * 16;
+    int t = blockIdx.x, ks = g;
+    TcItem x;
+    ColDesc col;
+    int E = 0;
+    // the group's next k-step: k-step ks of item t, or of a later item
+    auto settle = [&](bool fresh) -> bool {
+      for (; t < total; t += gridDim.x) {
+        if (fresh) x = item_at(B, t);
+        if (ks < x.ksteps) {
+          if (fresh) {
+            OpArgs a = B.a[x.cls];
+            a.m = x.m;
+            col = make_col(a, x.tile * kTcCols + ctile);
+            E = col_exponent(B, a, col, exps, pairing);
+          }
+          return true;
+        }
+        ks -= x.ksteps;
+        fresh = true;
+      }
+      return false;
+    };
+    long long w[16];
+    bool have = g < G && settle(true);
+    if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);
+    for (int it = g; have; it += G) {
+      const int s = it % S, use = it / S;
+      if (use > 0 && !(ok = __all_sync(0xffffffffu, pipe_wait(&empty[s], (use - 1) & 1, B.wait_ns)))) break;
+      unsigned char* xs = smtc + s * C::kStage + xoff;
+      const bool fscale = FI && E >= -78 && E <= 126;  // FMA-pipe slicing of float pairs
+      const f2 sc = f2_dup(pow2f(fscale ? 7 - E : 0)), sc3 = f2_dup(pow2f(fscale ? 31 - E : 0));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        unsigned int wd[4][kSlices];
+        if (fscale) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) digits_two(w[8 * h + 2 * i], w[8 * h + 2 * i + 1], sc, sc3, wd[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            unsigned int d0[kSlices], d1[kSlices];
+            digits_bf16(raw_fixed47<FI>(w[8 * h + 2 * i], E), d0);
+            digits_bf16(raw_fixed47<FI>(w[8 * h + 2 * i + 1], E), d1);
+#pragma unroll
+            for (int j = 0; j < kSlices; ++j) wd[i][j] = d0[j] | (d1[j] << 16);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kSlices; ++j)
+          *reinterpret_cast<uint4*>(xs + j * kTcXSlice + h * 128) = make_uint4(wd[0][j], wd[1][j], wd[2][j], wd[3][j]);
+      }
+      tc::fence_proxy_async();
+      bar_arrive(&xfull[s]);
+      ks += G;
+      have = settle(false);
+      if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);
+    }
+  } else if (warp >= kMmaWarp) {
+    if (warp == kLoadWarp && lane == 0) {
+      // the operator slices of a k-step; without the digit-sum-6 pairs the
+      // last five (digits 1..5 times 2^-16) stay in global memory
+      const uint32_t wcopy = B.sum6 ? C::kWBytes : (kTcWSlices - 5) * C::kWSlice;
+      int it = 0;
+      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+        const TcItem x = item_at(B, t);
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(B.W[x.cls].w + (size_t)x.m * B.W[x.cls].w_stride) +
+                                   (size_t)x.grp * x.ksteps * C::kWBytes;
+        for (int ks = 0; ks < x.ksteps; ++ks, ++it) {
+          const int s = it % S, use = it / S;
+          if (use > 0 && !(ok = pipe_wait(&empty[s], (use - 1) & 1, B.wait_ns))) break;
+          tc::bar_expect_tx(&wfull[s], wcopy);
+          tc::bulk_g2s(smtc + s * C::kStage + kTcXBytes, src + (size_t)ks * C::kWBytes, wcopy, &wfull[s]);
+        }
+      }
+      // every copy issued has landed before the CTA's memory goes, also after
+      // a wait gave up here or in another role (the long bound: these end)
+      for (int c = it > S ? it - S : 0; c < it; ++c) tc::bar_wait(&wfull[c % S], (c / S) & 1, kTcWaitNs);
+    }
+    if (warp == kMmaWarp && lane == 0) {
+      const uint32_t sbase = tc::smem_addr(smtc);
+      int it = 0, n = 0;
+      for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++n) {
+        const int ksteps = item_at(B, t).ksteps;
+        const int ai = n % A, ause = n / A;
+        if (ause > 0 && !(ok = pipe_wait(&accempty[ai], (ause - 1) & 1, B.wait_ns))) break;
+        const uint32_t ta = tm + ai * 256;
+        for (int ks = 0; ks < ksteps; ++ks, ++it) {
+          const int s = it % S;
+          const unsigned ph = (it / S) & 1;
+          ok = pipe_wait(&wfull[s], ph, B.wait_ns) && pipe_wait(&xfull[s], ph, B.wait_ns);
+          if (!ok) break;
+          tc::fence_after();
+          const uint32_t xa = sbase + s * C::kStage;
+          const uint64_t dx = tc::desc_kmajor(xa, 128, 256);
+          const uint64_t dw = tc::desc_kmajor(xa + kTcXBytes, 128, 256);
+          constexpr uint32_t ID = tc::idesc_bf16_f32(kTcCols, ROWS);
+          constexpr uint64_t XS = kTcXSlice >> 4, WS = C::kWSlice >> 4;  // slice strides, descriptor units
+          // digit-sum <= 4 pairs of input slice j: the operator slices 0..4-j
+          // are adjacent in shared memory and their accumulators acc_j..acc_4
+          // adjacent in TMEM, so up to 256 / ROWS of them go into one MMA of
+          // N = n ROWS (fewer re-reads of the input slice)
+          constexpr int kMerge = 256 / ROWS;
+#pragma unroll
+          for (int j = 0; j < 5; ++j)
+#pragma unroll
+            for (int i = 0; i + j <= 4; i += kMerge) {
+              const int nn = (5 - j - i) < kMerge ? (5 - j - i) : kMerge;
+              const uint32_t idn = tc::idesc_bf16_f32(kTcCols, nn * ROWS);
+              tc::mma(ta + (i + j) * ROWS, dx + j * XS, dw + i * WS, idn, (ks > 0 || j > 0) ? 1u : 0u);
+            }
+#pragma unroll
+          for (int i = 0; i < 6; ++i) tc::mma(ta + 4 * ROWS, dx + (5 - i) * XS, dw + (5 + i) * WS, ID, 1u);
+          if (B.sum6) {
+#pragma unroll
+            for (int i = 1; i < 6; ++i) tc::mma(ta + 4 * ROWS, dx + (6 - i) * XS, dw + (10 + i) * WS, ID, 1u);
+          }
+          tc::commit(&empty[s]);
+        }
+        if (ok) tc::commit(&accfull[ai]);
+      }
+      // the MMAs issued finish before the CTA's shared and tensor memory go,
+      // also after a wait gave up in some role (the long bound: these end)
+      tc::commit(&drained);
+      tc::bar_wait(&drained, 0, kTcWaitNs);
+    }
+  } else {
+    // epilogue warp: TMEM lanes 32 (warp % 4) .. + 31 (its columns), rows
+    // [h R, (h + 1) R) of every accumulator
+    constexpr int R = ROWS / 2, CH = 8;  // rows of a warp, rows at a time
+    const int q = warp & 3, h = warp >> 2;
+    const int ctile = q * 32 + lane;
+    float* rf = rowF[warp];
+    int n = 0;
+    for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
+      const TcItem x = item_at(B, t);
+      OpArgs a = B.a[x.cls];
+      a.m = x.m;
+      const ColDesc col = make_col(a, x.tile * kTcCols + ctile);
+      const int* rexp = B.W[x.cls].rowexp + (size_t)x.m * B.W[x.cls].rowexp_stride + x.grp * ROWS + h * R;
+      __syncwarp();
+      for (int i = lane; i < R; i += 32) rf[i] = pow2f(rexp[i]);
+      const ColScale cs(col_exponent(B, a, col, exps, pairing) - 14);
+      __syncwarp();
+      const int prow = min(a.g.P - x.grp * ROWS, ROWS);  // valid rows of this group
+      const int ai = n % A, ause = n / A;
+      ok = __all_sync(0xffffffffu, pipe_wait(&accfull[ai], ause & 1, B.wait_ns));
+      // the two warps of a column quarter leave together (they share barriers)
+      if (STAGE) ok = named_and(1 + q, 64, ok);
+      if (!ok) break;
+      tc::fence_after();
+      const uint32_t ta = tm + ai * 256 + ((uint32_t)(q * 32) << 16);
+      const int pend = min((h + 1) * R, prow);
+      long long* out = reinterpret_cast<long long*>(a.out);
+      const int prow0 = x.grp * ROWS;  // first row of the group within W
+      long long* o0 = out + col.out0;
+      const long long ors = a.g.out_rs;
+      long long* o1 = out + col.out1 - a.g.P0 * ors;
+      long long* stage = reinterpret_cast<long long*>(smtc + S * C::kStage) + (size_t)ctile * prow;
+      if (h * R >= pend) {
+        __syncwarp();
+        if (lane == 0) bar_arrive(&accempty[ai]);
+      }
+#pragma unroll 1
+      for (int p0 = h * R; p0 < pend; p0 += CH) {
+        uint32_t v[5][CH];
+#pragma unroll
+        for (int d = 0; d < 5; ++d) tc::ld_n(ta + d * ROWS + p0, v[d]);
+        tc::ld_wait(v[0]);
+#pragma unroll
+        for (int d = 1; d < 5; ++d) tc::tie(v[d]);
+        if (p0 + CH >= pend) {
+          // the accumulators are read: the next item may overwrite them
+          tc::fence_before();
+          __syncwarp();
+          if (lane == 0) bar_arrive(&accempty[ai]);
+        }
+        const int p = prow0 + p0;
+        const bool whole = p0 + CH <= pend && (p >= a.g.P0 || p + CH <= a.g.P0);
+        long long* o = (p >= a.g.P0 ? o1 : o0) + p * ors;  // a chunk within one output segment
+#pragma unroll
+        for (int j = 0; j < CH; j += 2) {
+          long long w0, w1;
+          fold_rows(v, j, rf + p0 - h * R + j, cs, w0, w1);
+          if (STAGE) {
+            if (p0 + j < pend) stage[p0 + j] = w0;
+            if (p0 + j + 1 < pend) stage[p0 + j + 1] = w1;
+          } else if (whole) {
+            if (col.valid) {
+              *o = w0;
+              o += ors;
+              *o = w1;
+              o += ors;
+            }
+          } else if (col.valid) {
+            if (p0 + j < pend) (p + j >= a.g.P0 ? o1 : o0)[(p + j) * ors] = w0;
+            if (p0 + j + 1 < pend) (p + j + 1 >= a.g.P0 ? o1 : o0)[(p + j + 1) * ors] = w1;
+          }
+        }
+      }
+      if constexpr (STAGE) {
+        // d_r: a quarter's outputs (32 columns of n_r rows each, out0 = c n_r)
+        // are one contiguous block, copied out with consecutive threads on
+        // consecutive words
+        named_sync(1 + q, 64);
+        const long long c0 = x.tile * kTcCols + q * 32;
+        const int words = (int)max(0ll, min(32ll, a.g.ncols - c0)) * prow;
+        const long long* from = reinterpret_cast<const long long*>(smtc + S * C::kStage) + (size_t)q * 32 * prow;
+        long long* dst = out + c0 * prow;
+        for (int e = h * 32 + lane; e < words; e += 64) dst[e] = from[e];
+        named_sync(1 + q, 64);
+      }
+    }
+  }
+  ok = __syncthreads_and(ok);
+  if (!ok && threadIdx.x == 0) atomicOr(flag, 2);
+  tc::fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    tc::fence_after();
+    tc::dealloc(tm, C::kTmemCols);
+  }
+}
+
+// The same products one item per CTA, for launches that do not fill the SMs:
+// their time is one item's latency, which more producer threads with fewer k
+// each shorten.  Producer warps (256 or 512 threads; one column and KQ = 8 or
+// 4 consecutive k of every k-step each) slice and, after the last k-step, run
+// the epilogue; one MMA warp copies the operator slices a stage ahead and
+// issues the products.
 template <int ROWS>
 struct TcCfg {
   static constexpr int kProd = ROWS == 48 ? 256 : 512;                 // producer threads
@@ -478,6 +986,7 @@ struct TcCfg {
   static_assert(kSmem <= 227 * 1024, "dynamic shared memory per CTA");
   static_assert(kStage % 1024 == 0, "stage alignment of the descriptors and bulk copies");
 };
+
 
 // Raw 64-bit words of N consecutive k of one column (zero outside K or in an
 // empty second segment; the sign of a negated segment applied on the bits).
@@ -498,108 +1007,30 @@ __device__ __forceinline__ void gather(const OpArgs& a, const ColDesc& d, int k0
   }
 }
 
-// (hi, lo) float pair, packed like the mixed path's internal storage, of
-// (a0 + a1 2^-8 + a2 2^-16 + a3 2^-24 + a4 2^-32) f1 f2 f3 (f1, f2, f3 powers of
-// two).  a0 + a1 2^-8 + a2 2^-16 + a3 2^-24 (exact values) is summed with
-// error-free transformations, so that the sum's only roundings are those of
-// the low words and of a4 2^-32 (below 2^-48 of |a0|); summing a3 2^-24 in
-// plain FP32 would cost about 2^-24 of it, more than the digit-sum-6 terms.
-__device__ __forceinline__ long long fold_pair(float a0, float a1, float a2, float a3, float a4, float f1,
-                                               float f2, float f3) {
-  ff r = two_sum(a0, fm(a1, 0.00390625f));
-  const ff q = two_sum(r.hi, fm(a2, 1.52587890625e-05f));
-  const ff v = two_sum(q.hi, fm(a3, 5.9604644775390625e-08f));
-  const float low = __fmaf_rn(a4, 2.3283064365386963e-10f, fa(fa(r.lo, q.lo), v.lo));
-  r = fast_two_sum(v.hi, low);
-  const float hi = fm(fm(fm(r.hi, f1), f2), f3), lo = fm(fm(fm(r.lo, f1), f2), f3);
-  return (long long)(((unsigned long long)__float_as_uint(lo) << 32) | __float_as_uint(hi));
-}
 
-// 2^k as a float, k clamped to the normal range
-__device__ __forceinline__ float pow2f(int k) {
-  return __int_as_float((max(-126, min(127, k)) + 127) << 23);
-}
-
-// Digit slices of a float pair x = hi + lo (|lo| < ulp(hi), |x| < 2^E) on the
-// FMA pipe.  Digit j has weight 2^(E - 7 - 8j) (the balanced base-256 digits
-// of round(x 2^(47 - E))).  For a float v and each j the exact steps
-//   d = rint(v / w_j) (one FFMA against 1.5 * 2^23),  v -= d w_j  (exact FFMA)
-// give balanced digits |d| <= 128 of v; the last digit rounds like the
-// fixed-point conversion.  lo contributes to digits 3..5 only (|lo| / w_2 < 1/2),
-// so digit j is d_j(hi) + d_j(lo), |.| <= 256, an exact BF16 value; it is the
-// same integer sum of weights as the rounded fixed point of hi plus that of lo.
-// Requires -78 <= E <= 126 (every weight and inverse weight a normal float).
-struct DigitScale {
-  float w[kSlices], inv[kSlices];
-};
-
-__device__ __forceinline__ DigitScale digit_scale(int E) {
-  DigitScale c;
-#pragma unroll
-  for (int j = 0; j < kSlices; ++j) {
-    c.w[j] = __int_as_float((E - 7 - 8 * j + 127) << 23);
-    c.inv[j] = __int_as_float((7 + 8 * j - E + 127) << 23);
-  }
-  return c;
-}
-
-__device__ __forceinline__ void digits_pair_f32(long long wbits, const DigitScale& c, float (&d)[kSlices]) {
-  constexpr float M = 12582912.0f;  // 1.5 * 2^23
-  float v = __int_as_float((int)(unsigned int)wbits);
-  float u = __int_as_float((int)(unsigned int)((unsigned long long)wbits >> 32));
-#pragma unroll
-  for (int j = 0; j < kSlices; ++j) {
-    d[j] = __fsub_rn(__fmaf_rn(v, c.inv[j], M), M);
-    if (j < kSlices - 1) v = __fmaf_rn(-d[j], c.w[j], v);
-  }
-#pragma unroll
-  for (int j = 3; j < kSlices; ++j) {
-    const float e = __fsub_rn(__fmaf_rn(u, c.inv[j], M), M);
-    if (j < kSlices - 1) u = __fmaf_rn(-e, c.w[j], u);
-    d[j] = __fadd_rn(d[j], e);
-  }
-}
-
-__device__ __forceinline__ void bar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(b)) : "memory");
-}
-
-// STAGE: the launch is d_r (one operator class, all rows in one group): the
-// epilogue stages the tile's outputs in shared memory and stores them as one
-// contiguous block.
 template <bool FI, int ROWS, bool STAGE = false>
-__global__ void __launch_bounds__(TcCfg<ROWS>::kThreads) k_op_tc(TcBatch B, const int* __restrict__ exps,
-                                                                 int pairing, int* __restrict__ flag) {
+__global__ void __launch_bounds__(TcCfg<ROWS>::kThreads)
+    k_op_tc(const __grid_constant__ TcBatch B, const int* __restrict__ exps, int pairing, int* __restrict__ flag) {
   using C = TcCfg<ROWS>;
   constexpr int S = C::kStages, KQ = C::kKQ;
-  extern __shared__ __align__(128) unsigned char smtc[];
+  extern __shared__ __align__(1024) unsigned char smtc[];
   __shared__ uint64_t xfull[S], wfull[S], empty[S], accf;
   __shared__ uint32_t tmem_base;
-  __shared__ float rowF[ROWS];  // 2^E_row
-  // operator class and azimuthal number of this CTA (blockIdx.y = class * nm + m)
-  const int cls = B.nclass > 1 ? (int)blockIdx.y / B.nm : 0;
-  OpArgs a = B.a[cls];
-  TcOp W = B.W[cls];
-  if ((long long)blockIdx.x >= B.tiles[cls] * W.ngroups) return;  // past this class's columns
+  __shared__ __align__(16) float rowF[ROWS];  // 2^E_row
+  const TcItem x = item_at(B, blockIdx.x);
+  OpArgs a = B.a[x.cls];
+  TcOp W = B.W[x.cls];
+  a.m = x.m;
+  W.w += (size_t)x.m * W.w_stride;
+  W.rowexp += (size_t)x.m * W.rowexp_stride;
+  const long long tile = x.tile;
+  const int grp = x.grp;
   const int tid = threadIdx.x;
   const bool producer = tid < C::kProd;
-  const long long tile = blockIdx.x / W.ngroups;
-  const int grp = (int)(blockIdx.x - tile * W.ngroups);
-  if (a.batched_m) {
-    a.m = (int)blockIdx.y - cls * B.nm;
-    W.w += (size_t)a.m * W.w_stride;
-    W.rowexp += (size_t)a.m * W.rowexp_stride;
-  }
   const int ctile = tid & (kTcCols - 1);        // column within the tile (producers)
   const int kq = (tid >> 7) * KQ;               // first k of this producer within a k-step
   const ColDesc col = make_col(a, tile * kTcCols + ctile);
-  int ce = exps[col.fld];
-  if (pairing) {
-    // slot pairs (f, f ^ 1), f >= kPairedFrom, of the same stacked shell
-    const int f = a.ns == 1 ? col.fld : col.fld / a.ns, sidx = col.fld - f * a.ns;
-    if (f >= kPairedFrom) ce = max(ce, exps[(f ^ 1) * a.ns + sidx]);
-  }
-  const int E = ce - 1022 + B.eoff;
+  const int E = col_exponent(B, a, col, exps, pairing);
   // the row exponents are needed only by the epilogue: loaded here, stored
   // to shared memory before the barrier that ends the main loop
   const int rexp = tid < ROWS ? W.rowexp[grp * ROWS + tid] : 0;
@@ -623,7 +1054,7 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads) k_op_tc(TcBatch B, cons
     // byte offset of this thread's row piece (column ctile, k kq..kq+KQ-1)
     const int xoff = (ctile >> 3) * 256 + (kq >> 3) * 128 + (ctile & 7) * 16 + (kq & 7) * 2;
     const bool fscale = E >= -78 && E <= 126;  // FMA-pipe slicing of float pairs
-    const DigitScale dsc = digit_scale(fscale ? E : 0);
+    const f2 sc = f2_dup(pow2f(fscale ? 7 - E : 0)), sc3 = f2_dup(pow2f(fscale ? 31 - E : 0));
     // The loads of the next k-step are issued after the arrive on the
     // current stage: the proxy fence and the arrive's release wait for every
     // load the thread has in flight, so loads issued before them would hold
@@ -641,13 +1072,10 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads) k_op_tc(TcBatch B, cons
       if (FI && fscale && ks * 16 + kq < a.g.K) {
 #pragma unroll
         for (int i = 0; i < KQ; i += 2) {
-          float f0[kSlices], f1[kSlices];
-          digits_pair_f32(cur[i], dsc, f0);
-          digits_pair_f32(cur[i + 1], dsc, f1);
-          // BF16 of an 8-bit integer float: its upper half
+          unsigned int d[kSlices];
+          digits_two(cur[i], cur[i + 1], sc, sc3, d);
 #pragma unroll
-          for (int j = 0; j < kSlices; ++j)
-            wd[j][i >> 1] = __byte_perm(__float_as_uint(f0[j]), __float_as_uint(f1[j]), 0x7632);
+          for (int j = 0; j < kSlices; ++j) wd[j][i >> 1] = d[j];
         }
       } else if (ks * 16 + kq < a.g.K) {
 #pragma unroll
@@ -756,31 +1184,24 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads) k_op_tc(TcBatch B, cons
     constexpr bool stage_out = STAGE;
     long long* out_tile = reinterpret_cast<long long*>(smtc);
     const uint32_t lane = tm + ((uint32_t)(((tid >> 5) & 3) * 32) << 16);
-    // 2^(E_col - 14) as two factors (the second is 1 unless E_col - 14 is
-    // below the float range, i.e. for outputs that underflow anyway)
-    const int ec = E - 14;
-    const float cf1 = pow2f(ec), cf2 = pow2f(ec - max(-126, min(127, ec)));
+    const ColScale cs(E - 14);
     // the group's rows of this thread's column, each folded result handed to
     // sink(row within the group, pair bits)
     auto rows_out = [&](auto&& sink) {
 #pragma unroll 1
       for (int p0 = g * R; p0 < (g + 1) * R && p0 < prow; p0 += 8) {
-        uint32_t v0[8], v1[8], v2[8], v3[8], v4[8];
-        tc::ld8(lane + 0 * ROWS + p0, v0);
-        tc::ld8(lane + 1 * ROWS + p0, v1);
-        tc::ld8(lane + 2 * ROWS + p0, v2);
-        tc::ld8(lane + 3 * ROWS + p0, v3);
-        tc::ld8(lane + 4 * ROWS + p0, v4);
-        tc::ld_wait(v0);
-        tc::tie(v1);
-        tc::tie(v2);
-        tc::tie(v3);
-        tc::tie(v4);
+        uint32_t v[5][8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (p0 + j < prow)
-            sink(p0 + j, fold_pair(__uint_as_float(v0[j]), __uint_as_float(v1[j]), __uint_as_float(v2[j]),
-                                   __uint_as_float(v3[j]), __uint_as_float(v4[j]), rowF[p0 + j], cf1, cf2));
+        for (int d = 0; d < 5; ++d) tc::ld_n(lane + d * ROWS + p0, v[d]);
+        tc::ld_wait(v[0]);
+#pragma unroll
+        for (int d = 1; d < 5; ++d) tc::tie(v[d]);
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+          long long w0, w1;
+          fold_rows(v, j, rowF + p0 + j, cs, w0, w1);
+          if (p0 + j < prow) sink(p0 + j, w0);
+          if (p0 + j + 1 < prow) sink(p0 + j + 1, w1);
         }
       }
     };
@@ -810,23 +1231,51 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads) k_op_tc(TcBatch B, cons
 // ---------------------------------------------------------------------------
 // Host side
 
+static int tiles_of(const OpArgs& a) { return (int)((a.g.ncols + kTcCols - 1) / kTcCols); }
+
+// Whether a launch of so many items takes the persistent kernel.  It pays from
+// a few items per SM on: with 96 rows (the one-item kernel holds one CTA per
+// SM) 297 / 322 / 1238 items take 27 / 35 / 96 us against 31 / 43 / 133; with 48
+// (two per SM) 470 items of d_theta + d_phi 24.3 against 25.7 us, 846 / 1128 items
+// of the projection 33 / 38 against 43 / 57, 1800 of d_r 57 against 65, but 450 of
+// d_r 19.6 against 17.4.
+static bool runs_persistent(const cffyn_shell* sh, int rows, long long items) {
+  return items > (rows == 48 ? 5 : 1) * (long long)sh->sm_count;
+}
+
 // Mixed path: one launch of the tcgen05 core over the classes of b (same row
-// group size, same input storage), grid = (max tiles x row groups,
-// classes x nm).
+// group size, same input storage).
 static int launch_batch(const cffyn_shell* sh, const TcBatch& b0, cudaStream_t st, int pairing, bool in_pairs,
                         const int* exps, int* flag = nullptr) {
   if (!flag) flag = sh->flag;
   TcBatch b = b0;
   b.wait_ns = sh->tc_wait_ns;
-  long long gx = 0;
-  for (int c = 0; c < b.nclass; ++c) gx = std::max(gx, b.tiles[c] * b.W[c].ngroups);
-  if (gx == 0) return CFFYN_OK;
-  const dim3 grid((unsigned)gx, (unsigned)(b.nclass * b.nm));
+  long long items = 0;
+  for (int c = 0; c < b.nclass; ++c) {
+    b.first[c] = (int)items;
+    items += (long long)b.tiles[c] * b.W[c].ngroups * (b.a[c].batched_m ? b.nm : 1);
+  }
+  if (items == 0) return CFFYN_OK;
+  if (items >= (1ll << 31)) {
+    set_error("operator launch of %lld tiles", items);
+    return CFFYN_EINVAL;
+  }
+  for (int c = b.nclass; c <= kMaxBatch; ++c) b.first[c] = (int)items;
+  const int rows = b.W[0].rows;
   // d_r (one class, one row group): the instance with the staged epilogue
-  const bool stage = b.nclass == 1 && b.a[0].kind == OP_R && b.W[0].ngroups == 1;
-#define CFFYN_LAUNCH_TC(R_, FI_, ST_) \
-  k_op_tc<FI_, R_, ST_><<<grid, TcCfg<R_>::kThreads, TcCfg<R_>::kSmem, st>>>(b, exps, pairing, flag)
-  if (b.W[0].rows == 48) {
+  const bool dr = b.nclass == 1 && b.a[0].kind == OP_R && b.W[0].ngroups == 1;
+  const bool persistent = runs_persistent(sh, rows, items);
+#define CFFYN_LAUNCH_TC(R_, FI_, ST_)                                                                        \
+  (persistent ? (void)(k_op_ws<FI_, R_, ST_><<<sh->sm_count, kWsThreads,                                      \
+                                               kRingStages<R_, ST_> * WsCfg<R_>::kStage + (ST_ ? out_bytes : 0), \
+                                               st>>>(b, exps, pairing, flag))                                \
+              : (void)(k_op_tc<FI_, R_, ST_><<<(unsigned)items, TcCfg<R_>::kThreads, TcCfg<R_>::kSmem, st>>>( \
+                    b, exps, pairing, flag)))
+  // the persistent instance keeps the staged outputs beside its ring
+  const int out_bytes = kTcCols * b.a[0].g.P * (int)sizeof(double);
+  const int ring = rows == 48 ? WsCfg<48>::kStage * kRingStages<48, true> : WsCfg<96>::kStage * kRingStages<96, true>;
+  const bool stage = dr && (!persistent || ring + out_bytes <= kTcMaxSmem);
+  if (rows == 48) {
     if (in_pairs)
       stage ? CFFYN_LAUNCH_TC(48, true, true) : CFFYN_LAUNCH_TC(48, true, false);
     else
@@ -864,7 +1313,7 @@ static int launch(const cffyn_shell* sh, const OpArgs& a, const double* W64, con
   memset(&b, 0, sizeof(b));
   b.a[0] = a;
   b.W[0] = *Wt;
-  b.tiles[0] = (a.g.ncols + kTcCols - 1) / kTcCols;
+  b.tiles[0] = tiles_of(a);
   b.nclass = 1;
   b.nm = (int)extra.y;
   b.eoff = eoff;
@@ -874,18 +1323,14 @@ static int launch(const cffyn_shell* sh, const OpArgs& a, const double* W64, con
 
 int set_op_smem_limits() {
   CF_CUDA(cudaFuncSetAttribute(k_op_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<true, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<48>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<false, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<48>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<true, 96>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<96>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<false, 96>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<96>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<true, 48, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               TcCfg<48>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<false, 48, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               TcCfg<48>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<true, 96, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               TcCfg<96>::kSmem));
-  CF_CUDA(cudaFuncSetAttribute(k_op_tc<false, 96, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               TcCfg<96>::kSmem));
+#define CFFYN_TC_INSTANCES(k) \
+  (const void*)k<true, 48>, (const void*)k<false, 48>, (const void*)k<true, 96>, (const void*)k<false, 96>, \
+      (const void*)k<true, 48, true>, (const void*)k<false, 48, true>, (const void*)k<true, 96, true>, \
+      (const void*)k<false, 96, true>
+  const void* tcs[] = {CFFYN_TC_INSTANCES(k_op_ws), CFFYN_TC_INSTANCES(k_op_tc)};
+#undef CFFYN_TC_INSTANCES
+  for (const void* f : tcs)
+    CF_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem));
   return CFFYN_OK;
 }
 
@@ -984,11 +1429,18 @@ int op_deriv_theta_phi(const cffyn_shell* sh, const double* in, double* out_th, 
   b.W[0] = sh->tDth2;
   b.a[1] = deriv_args(sh, 2, in, out_ph, nf);
   b.W[1] = sh->tDph;
-  for (int c = 0; c < 2; ++c) b.tiles[c] = (b.a[c].g.ncols + kTcCols - 1) / kTcCols;
+  for (int c = 0; c < 2; ++c) b.tiles[c] = tiles_of(b.a[c]);
   b.nclass = 2;
   b.nm = 1;
   b.sum6 = 1;
   return launch_batch(sh, b, st, 0, in_pairs, sh->exps);
+}
+
+// Whether the phi analysis of nf arrays runs on the persistent kernel: each of
+// its launches then fills the device by itself.
+bool op_dft_persistent(const cffyn_shell* sh, int nf) {
+  const long long tiles = ((long long)nf * sh->N * sh->n_r + kTcCols - 1) / kTcCols;
+  return sh->d.precision == CFFYN_MIXED && runs_persistent(sh, sh->tFan.rows, tiles * sh->tFan.ngroups);
 }
 
 static int op_rows(const cffyn_shell* sh, const double* in, double* out, int nb, int K, int P,
@@ -1065,7 +1517,7 @@ int op_project_scalar(const cffyn_shell* sh, const double* C, double* C2, cudaSt
     for (int c = 0; c < ncls; ++c) {
       bt.a[c] = cls[c];
       bt.W[c] = *Wt[c];
-      bt.tiles[c] = (cls[c].g.ncols + kTcCols - 1) / kTcCols;
+      bt.tiles[c] = tiles_of(cls[c]);
     }
     bt.nclass = ncls;
     bt.nm = nm;
@@ -1133,7 +1585,7 @@ int op_project(const cffyn_shell* sh, const double* C, double* C2, const int* sl
     for (int c = 0; c < ncls; ++c) {
       bt.a[c] = cls[c];
       bt.W[c] = *Wt[c];
-      bt.tiles[c] = (cls[c].g.ncols + kTcCols - 1) / kTcCols;
+      bt.tiles[c] = tiles_of(cls[c]);
     }
     bt.nclass = ncls;
     bt.nm = nm;

@@ -39,19 +39,26 @@ __device__ __forceinline__ void bar_init(uint64_t* b, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
 }
 
+// One poll of the phase of barrier a.
+__device__ __forceinline__ bool bar_try(uint32_t a, unsigned parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(a), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Waits until the phase with the given parity of barrier b has completed.
-// Gives up (returns false) after limit_ns nanoseconds or 2^26 polls.
+// Gives up (returns false) after limit_ns nanoseconds or 2^26 polls.  The
+// timer is read only when the first poll fails.
 __device__ __forceinline__ bool bar_wait(uint64_t* b, unsigned parity, unsigned long long limit_ns) {
   const uint32_t a = smem_addr(b);
+  if (bar_try(a, parity)) return true;
   const unsigned long long t0 = now_ns();
   for (int it = 0; it < (1 << 26); ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (ok) return true;
+    if (bar_try(a, parity)) return true;
     if (now_ns() - t0 > limit_ns) return false;
   }
   return false;
@@ -130,12 +137,26 @@ __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 
 // 8 consecutive 32-bit TMEM columns of this thread's lane.  Not waited on.
-__device__ __forceinline__ void ld8(uint32_t taddr, uint32_t (&r)[8]) {
+__device__ __forceinline__ void ld_n(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                  "=r"(r[7])
                : "r"(taddr)
                : "memory");
+}
+
+// 4 consecutive 32-bit TMEM columns of this thread's lane.  Not waited on.
+__device__ __forceinline__ void ld_n(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void ld_wait(uint32_t (&r)[4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+}
+__device__ __forceinline__ void tie(uint32_t (&r)[4]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
 }
 
 #define CFFYN_TIE8(r) \

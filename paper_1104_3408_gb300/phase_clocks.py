@@ -1,15 +1,15 @@
-"""Per-block phase clocks of the tensor-core operator kernel (a diagnostic).
+"""Per-CTA phase clocks of the tensor-core operator kernel (a diagnostic).
 
-Builds a copy of the library whose k_op_tc records, for every block of the
-d_theta + d_phi launch, SM clock64 intervals of its phases (set-up, the MMA
-thread's waits for operator copies, for the producers' slices, its issue of
-the products and its refill waits, the producers' waits for free stages and
-their loop, the products' completion and the epilogue), runs RK4 steps of the
-33 x 48 x 96 shell with it, and prints the phase means over the blocks of
-the last such launch.  The copy lives under the package's build folder; the
-library itself is unchanged.
+Builds a copy of the library whose k_op_tc sums, for every CTA of the
+d_theta + d_phi launch, SM clock64 intervals of each role: the MMA thread's
+waits (operator copies, slices, accumulators) and its issue, a producer warp's
+wait for a free stage, slicing and load issue, an epilogue warp's wait for
+products, its reading of the accumulators and the rest of its stores.  Runs
+RK4 steps of a shell with it and prints the means over the CTAs of the last
+such launch, per work item.  The copy lives under the package's build folder;
+the library itself is unchanged.
 
-    python -m paper_1104_3408_gb300.phase_clocks [--mhz F]
+    python -m paper_1104_3408_gb300.phase_clocks [--mhz F] [--shape NR,NTHETA]
 
 (F: the SM clock used to turn cycles into microseconds, default 2070.)
 """
@@ -25,32 +25,56 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 OUT = os.path.join(PKG, "_lib", "phase_clocks")
 
-NAMES = ["mma: wait for operator copies", "mma: wait for slices", "mma: issue of the products",
-         "mma: wait to refill (previous k-step done)", "mma: end of its loop", "mma: first k-step ready",
-         "products done", "end of epilogue", "producer 0: wait for free stages", "producer 0: its loop",
-         "producer 0: loop + products done", "set-up"]
+NAMES = ["mma: wait for operator copies", "mma: wait for slices", "mma: wait for accumulators",
+         "mma: issue of the products", "mma: whole loop", "producer: wait for a free stage", "producer: slicing",
+         "producer: next k-step's loads issued", "epilogue: wait for products", "epilogue: accumulators read",
+         "epilogue: last rows folded and stored", "set-up"]
 
 
 # (text of the kernel, text with the clocks) pairs applied to a copy of csrc/ops.cu
 _PATCHES = [
-    ('// STAGE: the launch is d_r (one operator class, all rows in one group): the',
-     '__device__ unsigned long long g_instr[4096][16];\n// STAGE: the launch is d_r (one operator class, all rows in one group): the'),
-    ('  using C = TcCfg<ROWS>;\n  constexpr int S = C::kStages, KQ = C::kKQ;\n  extern __shared__ __align__(128) unsigned char smtc[];',
-     '  using C = TcCfg<ROWS>;\n  constexpr int S = C::kStages, KQ = C::kKQ;\n  const unsigned long long c_entry = clock64();\n  unsigned long long ins[16] = {0};\n  extern __shared__ __align__(128) unsigned char smtc[];'),
-    ('  const int ksteps = W.ksteps;\n  bool ok = true;\n',
-     '  const int ksteps = W.ksteps;\n  bool ok = true;\n  const unsigned long long c_setup = clock64();\n'),
-    ('      if (ks >= S && ok) ok = pipe_wait(&empty[s], ((ks - S) / S) & 1, B.wait_ns);',
-     '      const unsigned long long pw0 = clock64();\n      if (ks >= S && ok) ok = pipe_wait(&empty[s], ((ks - S) / S) & 1, B.wait_ns);\n      ins[8] += clock64() - pw0;'),
-    ('    if (ok) ok = pipe_wait(&accf, 0, B.wait_ns);\n  } else if (tid == C::kProd) {',
-     '    ins[9] = clock64() - c_setup;\n    if (ok) ok = pipe_wait(&accf, 0, B.wait_ns);\n    ins[10] = clock64() - c_setup;\n  } else if (tid == C::kProd) {'),
-    ('      ok = pipe_wait(&wfull[s], (ks / S) & 1, B.wait_ns) && pipe_wait(&xfull[s], (ks / S) & 1, B.wait_ns);\n      if (!ok) break;',
-     '      const unsigned long long m0 = clock64();\n      ok = pipe_wait(&wfull[s], (ks / S) & 1, B.wait_ns);\n      const unsigned long long m1 = clock64();\n      ok = ok && pipe_wait(&xfull[s], (ks / S) & 1, B.wait_ns);\n      const unsigned long long m2 = clock64();\n      ins[0] += m1 - m0;\n      ins[1] += m2 - m1;\n      if (ks == 0) ins[5] = m2 - c_setup;\n      if (!ok) break;'),
-    ('      tc::commit(&empty[s]);\n      // refill the stage of k-step ks - 1 with the operator of k-step ks - 1 + S\n      if (ks >= 1 && copied < ksteps) {\n        const int sp = (ks - 1) % S;\n        ok = pipe_wait(&empty[sp], ((ks - 1) / S) & 1, B.wait_ns);',
-     '      tc::commit(&empty[s]);\n      const unsigned long long m3 = clock64();\n      ins[2] += m3 - m2;\n      // refill the stage of k-step ks - 1 with the operator of k-step ks - 1 + S\n      if (ks >= 1 && copied < ksteps) {\n        const int sp = (ks - 1) % S;\n        ok = pipe_wait(&empty[sp], ((ks - 1) / S) & 1, B.wait_ns);\n        ins[3] += clock64() - m3;'),
-    ('    tc::commit(&accf);\n    if (!ok) {',
-     '    tc::commit(&accf);\n    ins[4] = clock64() - c_setup;\n    tc::bar_wait(&accf, 0, kTcWaitNs);\n    ins[6] = clock64() - c_setup;\n    if (!ok) {'),
-    ('  tc::fence_before();\n  __syncthreads();\n  if (tid >= C::kProd) {\n    tc::fence_after();\n    tc::dealloc(tm, C::kTmemCols);\n  }\n}',
-     '  tc::fence_before();\n  __syncthreads();\n  if (B.nclass == 2 && blockIdx.x < 2048) {\n    const int rec = (int)(blockIdx.y * 2048 + blockIdx.x) % 4096;\n    if (tid == C::kProd) {\n      ins[7] = clock64() - c_setup;\n      ins[11] = c_setup - c_entry;\n      for (int q = 0; q < 8; ++q) g_instr[rec][q] = ins[q];\n      g_instr[rec][11] = ins[11];\n      g_instr[rec][12] = ksteps;\n    }\n    if (tid == 0) {\n      g_instr[rec][8] = ins[8];\n      g_instr[rec][9] = ins[9];\n      g_instr[rec][10] = ins[10];\n    }\n  }\n  if (tid >= C::kProd) {\n    tc::fence_after();\n    tc::dealloc(tm, C::kTmemCols);\n  }\n}\n\nextern "C" __attribute__((visibility("default"))) int cffyn_instr_read(unsigned long long* host) {\n  return (int)cudaMemcpyFromSymbol(host, g_instr, sizeof(g_instr));\n}'),
+    ("// STAGE: the launch is d_r (one operator class, all rows in one group): the",
+     "__device__ unsigned long long g_instr[1024][16];\n#define CK clock64()\n"
+     "// STAGE: the launch is d_r (one operator class, all rows in one group): the"),
+    ("  const int total = B.first[B.nclass];\n",
+     "  const int total = B.first[B.nclass];\n  const long long c_entry = CK;\n  long long ins[12] = {0};\n"),
+    ("  const uint32_t tm = tmem_base;\n", "  const uint32_t tm = tmem_base;\n  const long long c_setup = CK;\n"),
+    ("      if (use > 0 && !(ok = __all_sync", "      const long long p0_ = CK;\n      if (use > 0 && !(ok = __all_sync"),
+    ("      unsigned char* xs = smtc + s * C::kStage + xoff;\n",
+     "      unsigned char* xs = smtc + s * C::kStage + xoff;\n      const long long p1_ = CK;\n"),
+    ("      bar_arrive(&xfull[s]);\n", "      bar_arrive(&xfull[s]);\n      const long long p2_ = CK;\n"),
+    ("      if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);\n    }\n",
+     "      if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);\n      ins[5] += p1_ - p0_;\n      ins[6] += p2_ - p1_;\n"
+     "      ins[7] += CK - p2_;\n    }\n"),
+    ("        const int ai = n % A, ause = n / A;\n        if (ause > 0",
+     "        const int ai = n % A, ause = n / A;\n        const long long a0_ = CK;\n        if (ause > 0"),
+    ("        const uint32_t ta = tm + ai * 256;\n        for (int ks",
+     "        const uint32_t ta = tm + ai * 256;\n        ins[2] += CK - a0_;\n        for (int ks"),
+    ("          ok = pipe_wait(&wfull[s], ph, B.wait_ns) && pipe_wait(&xfull[s], ph, B.wait_ns);\n",
+     "          const long long m0_ = CK;\n          ok = pipe_wait(&wfull[s], ph, B.wait_ns);\n          const long long m1_ = CK;\n"
+     "          ok = ok && pipe_wait(&xfull[s], ph, B.wait_ns);\n          const long long m2_ = CK;\n"
+     "          ins[0] += m1_ - m0_;\n          ins[1] += m2_ - m1_;\n"),
+    ("          tc::commit(&empty[s]);\n", "          tc::commit(&empty[s]);\n          ins[3] += CK - m2_;\n"),
+    ("      tc::bar_wait(&drained, 0, kTcWaitNs);\n", "      tc::bar_wait(&drained, 0, kTcWaitNs);\n      ins[4] = CK - c_setup;\n"),
+    ("      ok = __all_sync(0xffffffffu, pipe_wait(&accfull[ai], ause & 1, B.wait_ns));\n",
+     "      const long long e0_ = CK;\n      ok = __all_sync(0xffffffffu, pipe_wait(&accfull[ai], ause & 1, B.wait_ns));\n"
+     "      long long e1_ = CK, e2_ = 0;\n"),
+    ("          // the accumulators are read: the next item may overwrite them\n",
+     "          e2_ = CK;\n          // the accumulators are read: the next item may overwrite them\n"),
+    ("      if constexpr (STAGE) {\n        // d_r: a quarter",
+     "      ins[8] += e1_ - e0_;\n      if (e2_) ins[9] += e2_ - e1_, ins[10] += CK - e2_;\n"
+     "      if constexpr (STAGE) {\n        // d_r: a quarter"),
+    ("  ok = __syncthreads_and(ok);\n",
+     "  if (!STAGE && B.sum6 && B.nclass == 2 && lane == 0) {\n    const int lo = warp == kMmaWarp ? 0 : warp == kProdWarp0 ? 5 : warp == 0 ? 8 : 12;\n"
+     "    const int hi = warp == kMmaWarp ? 5 : warp == kProdWarp0 ? 8 : warp == 0 ? 11 : 12;\n"
+     "    for (int q = 0; q < 11; ++q)\n      if (q >= lo && q < hi) g_instr[blockIdx.x][q] = (unsigned long long)ins[q];\n"
+     "    if (warp == 0) {\n      g_instr[blockIdx.x][11] = (unsigned long long)(c_setup - c_entry);\n"
+     "      g_instr[blockIdx.x][12] = (total - blockIdx.x + gridDim.x - 1) / gridDim.x;\n    }\n  }\n"
+     "  ok = __syncthreads_and(ok);\n"),
+    ("// ---------------------------------------------------------------------------\n// Host side\n",
+     "extern \"C\" __attribute__((visibility(\"default\"))) int cffyn_instr_read(unsigned long long* host) {\n"
+     "  return (int)cudaMemcpyFromSymbol(host, g_instr, sizeof(g_instr));\n}\n"
+     "// ---------------------------------------------------------------------------\n// Host side\n"),
 ]
 
 
@@ -98,6 +122,7 @@ def build():
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--mhz", type=float, default=2070.0)
+    ap.add_argument("--shape", default="33,48", help="n_r,n_theta")
     args = ap.parse_args()
     if ROOT not in sys.path:
         sys.path.insert(0, ROOT)
@@ -107,23 +132,24 @@ def main():
     from . import cffyn, inputs
     lib = cffyn.load(build())
     lib.cffyn_instr_read.argtypes = [ctypes.c_void_p]
-    n_r, N, J, L = 33, 48, 96, 46
+    n_r, N = (int(v) for v in args.shape.split(","))
+    J, L = 2 * N, N - 2
     sh = cffyn.Shell(n_r, N, J, 1.8, 11.0, L)
     u = torch.from_numpy(inputs.kerr_schild_state(n_r, N, J, 1.8, 11.0, amp=1e-4, ell=4, seed=0)).cuda()
     sh.init_gauge_from_state(u)
     for _ in range(3):
         sh.rk4_step(u, 0.0, 1)
     torch.cuda.synchronize()
-    buf = np.zeros((4096, 16), dtype=np.uint64)
+    buf = np.zeros((1024, 16), dtype=np.uint64)
     if lib.cffyn_instr_read(buf.ctypes.data) != 0:
         raise RuntimeError("reading the phase clocks failed")
     rec = buf[buf[:, 12] > 0].astype(np.float64)
-    us = rec / args.mhz
-    print(f"d_theta + d_phi launch of the {n_r}x{N}x{J} shell: {len(rec)} blocks, "
-          f"{int(rec[0, 12])} k-steps each; microseconds at {args.mhz:.0f} MHz (mean, p10, p90)")
+    items = rec[:, 12]
+    print(f"d_theta + d_phi launch of the {n_r}x{N}x{J} shell: {len(rec)} CTAs, {items.mean():.2f} items each; "
+          f"microseconds at {args.mhz:.0f} MHz per item (mean, p10, p90)")
     for q, nm in enumerate(NAMES):
-        print(f"{nm:45s} {us[:, q].mean():7.2f} {np.percentile(us[:, q], 10):7.2f} "
-              f"{np.percentile(us[:, q], 90):7.2f}")
+        us = rec[:, q] / args.mhz / (items if q < 11 else 1.0)
+        print(f"{nm:45s} {us.mean():7.2f} {np.percentile(us, 10):7.2f} {np.percentile(us, 90):7.2f}")
     sh.destroy()
 
 
