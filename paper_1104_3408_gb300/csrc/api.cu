@@ -729,10 +729,14 @@ static int enqueue_step(cffyn_shell* sh, double* u, double dt, cudaStream_t st) 
 extern "C++" {
 namespace cffyn {
 
-// One RK4 step enqueued on st without trace marks (a branch of a batch graph).
-int enqueue_step_branch(cffyn_shell* sh, double* u, double dt, cudaStream_t st) {
+// One RK4 step enqueued on st without trace marks (a branch of a batch graph);
+// beside: the points of the batch's other branches.
+int enqueue_step_branch(cffyn_shell* sh, double* u, double dt, cudaStream_t st, long long beside) {
   auto run = [](int, auto&& fn) -> int { return fn(); };
-  return step_sequence(sh, u, dt, st, run, true);
+  sh->beside = beside;
+  const int rc = step_sequence(sh, u, dt, st, run, true);
+  sh->beside = 0;
+  return rc;
 }
 
 // The pieces of a step for nested shells (no trace marks): stage s's

@@ -23,7 +23,7 @@
 #include "common.cuh"
 
 namespace cffyn {
-int enqueue_step_branch(cffyn_shell*, double*, double, cudaStream_t);
+int enqueue_step_branch(cffyn_shell*, double*, double, cudaStream_t, long long);
 int enqueue_step_prologue(cffyn_shell*, double*, cudaStream_t);
 int step_flag_status(int);
 int check_step_ready(const cffyn_shell*);
@@ -340,7 +340,10 @@ int cffyn_batch_rk4_step(cffyn_batch* b, double* const* u, const double* dt, int
     if ((rc = capture_branches(b, &b->step, [&](int i, cudaStream_t s) {
            const Unit& un = b->units[i];
            const int m0 = un.members[0];
-           return enqueue_step_branch(un.handle(b->sh), un.stack ? un.U : u[m0], dts[m0], s);
+           cffyn_shell* k = un.handle(b->sh);
+           long long beside = -(long long)P_all(k);
+           for (const Unit& o : b->units) beside += (long long)P_all(o.handle(b->sh));
+           return enqueue_step_branch(k, un.stack ? un.U : u[m0], dts[m0], s, beside);
          }))) {
       free_graphs(b);
       return rc;

@@ -72,6 +72,8 @@ struct cffyn_shell {
   size_t bytes = 0;
   int device = 0;
   int sm_count = 1;             // SMs of the device: CTAs of a persistent launch
+  long long beside = 0;         // points advanced beside this handle's launches while they are captured
+                                // (the other classes of a batch); 0 otherwise
 
   // grid (device)
   double *r = nullptr, *sth = nullptr, *cth = nullptr, *sph = nullptr, *cph = nullptr;

@@ -593,6 +593,245 @@ __global__ void __launch_bounds__(128, 9) k_reconstruct(const double* __restrict
   if (bad) atomicOr(flag, 1);
 }
 
+// ---------------------------------------------------------------------------
+// k_reconstruct for few points (recon_shared): 32 points per block with eight
+// warps, each warp a share of every point's tensor components.  As one thread
+// per tensor group the rank-3 group's 18 components are one chain of 14 us
+// (stages 1-3) to 31 us (last stage) however few points there are; shared out it
+// takes 9 to 17 (13 x 9 x 18).  The three warps of the rank-3 tensor exchange
+// their legs through shared memory, [slot][point].  Same results.
+//
+// Shares: 0..2 the legs of group 7 (six components each), 3 group 6 (nine), 4 and
+// 5 groups 4 and 5 (six each), 6 groups 1 and 2, 7 groups 3 and 0, 8 and 9 the
+// gauge groups.
+template <class T>
+struct PointScratch {
+  T* s;  // this point's column
+  __device__ __forceinline__ T& operator()(int v) const { return s[v * 32]; }
+};
+constexpr int kShares = 8;  // warps of a block
+
+// barrier over the first nthreads threads that name it
+__device__ __forceinline__ void bar_part(int id, int nthreads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// The point and share of a thread.  blockIdx.y = 1 (54/58-field states): the
+// gauge groups, ng per point, one warp each; `share` is then 8 + group.
+// p: the point, for a spare thread of the last block the last point; live:
+// whether the thread's results are stored.
+struct Share {
+  int share;
+  long long p;
+  bool live, any;
+};
+__device__ __forceinline__ Share share_of(const Geo& geo) {
+  Share x;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  long long blk = blockIdx.x;
+  x.share = w;
+  if (blockIdx.y == 1) {
+    const int ng = (geo.nv - 50) / 4;
+    x.share = 8 + w % ng;
+    blk = blockIdx.x * (long long)(kShares / ng) + w / ng;
+  }
+  const long long q = blk * 32 + lane;
+  x.live = q < geo.P;
+  x.any = blk * 32 < geo.P;
+  x.p = x.live ? q : geo.P - 1;
+  return x;
+}
+
+// The rank-3 group, warp w of three: the pair part Trot_A of triad leg
+// A = w back to Cartesian (X_A, slots 6 A + q, q: rr, r1, r2, 11, 12, 22), then
+// the components with derivative leg a = w: field 24 + 10 w + q to emit(q, value).
+template <class T, class Emit>
+__device__ __forceinline__ void reconstruct_rank3(int w, PointScratch<T> sc, const double* __restrict__ sp, long long P,
+                                                  long long p, const Triad<T>& t, Emit&& emit) {
+  const T half = S<T>::c(0.5);
+  auto in = [&](int slot) { return ld<T, kIn<T>>(sp, P, p, slot); };
+  T pr, pmb, prm0, prm1, pmm0, pmm1;
+  if (w == 0) {
+    pr = in(SLOT_R0(10));
+    pmb = in(SLOT_R0(11));
+    prm0 = in(SLOT_C1(7));
+    prm1 = in(SLOT_C1(7) + 1);
+    pmm0 = in(SLOT_C2(3));
+    pmm1 = in(SLOT_C2(3) + 1);
+  } else {
+    pr = in(SLOT_C1(8) + w - 1);
+    pmb = in(SLOT_C1(9) + w - 1);
+    // X = (m; rm) = P^th + i P^ph, Y = (m; r mbar) = conj(P^th) + i conj(P^ph)
+    const T xr = in(SLOT_C2(4)), xi = in(SLOT_C2(4) + 1), yr = in(SLOT_R0(14)), yi = in(SLOT_R0(15));
+    // X' = (m; mm) = P^th + i P^ph, Z = (mbar; mm) = P^th - i P^ph
+    const T mr = in(SLOT_C3), mi = in(SLOT_C3 + 1), zr = in(SLOT_C1(10)), zi = in(SLOT_C1(10) + 1);
+    if (w == 1) {
+      prm0 = half * (xr + yr);
+      prm1 = half * (xi - yi);
+      pmm0 = half * (mr + zr);
+      pmm1 = half * (mi + zi);
+    } else {
+      prm0 = half * (xi + yi);
+      prm1 = half * (yr - xr);
+      pmm0 = half * (mi - zi);
+      pmm1 = half * (zr - mr);
+    }
+  }
+  {
+    T Trot[3][3], X[3][3];
+    Trot[0][0] = pr;
+    Trot[0][1] = prm0;
+    Trot[0][2] = prm1;
+    Trot[1][1] = half * (pmb + pmm0);
+    Trot[1][2] = half * pmm1;
+    Trot[2][2] = half * (pmb - pmm0);
+    unrot_sym(t, Trot, X);
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+      for (int c = b; c < 3; ++c) sc(6 * w + SI(b + 1, c + 1) - 4) = X[b][c];
+  }
+  bar_part(1, 96);
+  const T r0 = triad_col_el(t, 0, w), r1 = triad_col_el(t, 1, w), r2 = triad_col_el(t, 2, w);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) emit(q, r0 * sc(q) + r1 * sc(6 + q) + r2 * sc(12 + q));
+}
+
+// Output fields of each share.
+__host__ __device__ constexpr bool in_share(int W, int f) {
+  return W < 3  ? (f >= 24 + 10 * W && f < 30 + 10 * W)
+       : W == 3 ? (f >= 20 && f < 50 && (f % 10) >= 1 && (f % 10) <= 3)
+       : W == 4 ? (f >= 4 && f <= 9)
+       : W == 5 ? (f >= 14 && f <= 19)
+       : W == 6 ? ((f >= 1 && f <= 3) || (f >= 11 && f <= 13))
+       : W == 7 ? (f == 20 || f == 30 || f == 40 || f == 0 || f == 10)
+       : W == 8 ? (f >= 50 && f < 54)
+                : (f >= 54 && f < 58);
+}
+
+// State words of one field that its update needs, loaded ahead of the update.
+template <class T, int KIND>
+struct StateWords {
+  T base, acc;  // KIND 1: base of U, accumulator; KIND 2: accumulator
+  double un;    // KIND 2: the state
+};
+
+template <class T, int KIND>
+struct StageUpdate {
+  double *dst, *u, *U, *kacc, *uf;
+  long long P, p;
+  int stage;  // 0..3
+  bool live, bad;
+  T cU, sixth;
+  using SI_ = Store<T, kIn<T>>;
+  static constexpr bool kPair = kIn<T>;  // mixed path: the step's initial state also as pairs in uf
+
+  __device__ __forceinline__ StateWords<T, KIND> fetch(int f) const {
+    const long long o = (long long)f * P + p;
+    StateWords<T, KIND> x;
+    if (KIND == 1) {
+      // stage state: FP64 sum on the FP64 path, double-float on the mixed path
+      x.base = kPair ? SI_::ld(uf, o) : S<T>::c(__ldg(u + o));
+      if (stage != 0) x.acc = SI_::ld(kacc, o);
+    } else if (KIND == 2) {
+      x.un = __ldg(u + o);
+      x.acc = SI_::ld(kacc, o);
+    }
+    return x;
+  }
+  // (read-only loads, free to move ahead of other fields' stores: a word is
+  // read by the thread that writes it, before it writes)
+  // the update of field f with its right-hand side k
+  __device__ __forceinline__ void put(int f, T k, const StateWords<T, KIND>& x) {
+    const long long o = (long long)f * P + p;
+    if (KIND == 0) {
+      if (!live) return;
+      Store<T, false>::st(dst, o, k);
+      if (kPair && uf) SI_::st(uf, o, k);
+    } else if (KIND == 1) {
+      bad |= !finite_s(k);
+      const T acc = stage == 0 ? k : x.acc + (k + k), un = x.base + cU * k;
+      if (!live) return;
+      SI_::st(kacc, o, acc);
+      SI_::st(U, o, un);
+    } else {
+      bad |= !finite_s(k);
+      const double un = x.un + S<T>::to_double(sixth * (x.acc + k));
+      if (!live) return;
+      u[o] = un;
+      if (kPair && uf) SI_::st(uf, o, S<T>::c(un));
+    }
+  }
+};
+
+// Latency-bound (a few dependent loads and stores per field): 32 warps per SM
+// of at most 64 registers, the state words of the rank-3 legs in flight over
+// their exchange.
+template <class T, int KIND>
+__global__ void __launch_bounds__(32 * kShares, 4)
+    k_reconstruct_shared(const double* __restrict__ sp, double* __restrict__ dst, Geo geo, int mode, double* __restrict__ u,
+                  double* __restrict__ U, double* __restrict__ kacc, double* __restrict__ uf, double dt,
+                  int* __restrict__ flag) {
+  __shared__ T sm[kRecSlots * 32];  // X_A of the rank-3 tensor (3 x 6)
+  const Share x = share_of(geo);
+  if (!x.any) return;
+  const int stage = KIND == 0 ? 0 : (mode - 1) % 4;  // 0..3 for modes 1..8; KIND 2 is stage 3
+  StageUpdate<T, KIND> up{dst,   u,     U,     kacc,  uf, geo.P, x.p,
+                          stage, x.live, false, S<T>::c(stage == 2 ? dt : 0.5 * dt), S<T>::c(dt / 6.0)};
+  if (mode <= 4) {
+    const int i = (int)((x.p / geo.n_r) % geo.N);
+    const int jj = (int)((x.p / ((long long)geo.n_r * geo.N)) % geo.J);
+    const Triad<T> t = triad_at<T>(geo, i, jj);
+    auto emit = [&](int f, T k) { up.put(f, k, up.fetch(f)); };
+    auto group = [&](int g) { reconstruct_group<T>(g, Scratch<T>{nullptr}, sp, geo.P, x.p, t, emit); };
+    switch (x.share) {
+      case 0:
+      case 1:
+      case 2: {
+        StateWords<T, KIND> words[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) words[q] = up.fetch(24 + 10 * x.share + q);
+        reconstruct_rank3<T>(x.share, PointScratch<T>{sm + (threadIdx.x & 31)}, sp, geo.P, x.p, t,
+                             [&](int q, T k) { up.put(24 + 10 * x.share + q, k, words[q]); });
+        break;
+      }
+      case 3: group(6); break;
+      case 4: group(4); break;
+      case 5: group(5); break;
+      case 6:
+        group(1);
+        group(2);
+        break;
+      case 7:
+        group(3);
+        group(0);
+        break;
+      default: group(x.share); break;
+    }
+  } else {
+#define CFFYN_COPY(W)                                                 \
+  case W: {                                                           \
+    _Pragma("unroll") for (int f = 0; f < kMaxNv; ++f) if (in_share(W, f)) \
+        up.put(f, ld<T, kIn<T>>(sp, geo.P, x.p, f), up.fetch(f));     \
+    break;                                                            \
+  }
+    switch (x.share) {
+      CFFYN_COPY(0)
+      CFFYN_COPY(1)
+      CFFYN_COPY(2)
+      CFFYN_COPY(3)
+      CFFYN_COPY(4)
+      CFFYN_COPY(5)
+      CFFYN_COPY(6)
+      CFFYN_COPY(7)
+      CFFYN_COPY(8)
+      CFFYN_COPY(9)
+    }
+#undef CFFYN_COPY
+  }
+  if (up.bad) atomicOr(flag, 1);
+}
+
 // Spherical -> Cartesian derivatives: D[3][nf][P] -> out[3][nf][P] (FP64
 // arithmetic; D and out in the given storages).  Setup and API paths only.
 // One thread per point: the Jacobian (FP64 divisions) is formed once and
@@ -723,6 +962,11 @@ int pw_decompose(const cffyn_shell* sh, const double* in, double* out, bool in_p
   return CFFYN_OK;
 }
 
+// Whether a point's components are shared out over eight warps: up to one block of
+// 128 points per SM (stages 1-3 / last stage, us: 8704 points 15 / 24 against 31 /
+// 38, 28800 points 27 / 45 against 31 / 41, 152064 points 110 / 177 against 71 / 101).
+static bool recon_shared(const cffyn_shell* sh, unsigned nb) { return nb + sh->beside / 128 <= sh->sm_count; }
+
 // dst (mode 0) is an FP64 array; uf (mixed path): the step's initial state as
 // pairs, read by stages 1-3 and written by the last stage and by mode 0
 int pw_reconstruct(const cffyn_shell* sh, const double* sp, double* dst, int mode, double* u, double* U,
@@ -731,21 +975,18 @@ int pw_reconstruct(const cffyn_shell* sh, const double* sp, double* dst, int mod
   const dim3 grid(blocks_for(g.P, 128), kGroups + sh->ng);
   // kernel instance by stage kind: 0 filtered result, 1 stages 1-3, 2 last stage
   const int kind = (mode == 0 || mode == 9) ? 0 : ((mode - 1) % 4 == 3 ? 2 : 1);
-  if (sh->d.precision == CFFYN_MIXED) {
-    if (kind == 0)
-      k_reconstruct<ff, false, 0><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, uf, dt, flag);
-    else if (kind == 1)
-      k_reconstruct<ff, false, 1><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, uf, dt, flag);
-    else
-      k_reconstruct<ff, false, 2><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, uf, dt, flag);
-  } else {
-    if (kind == 0)
-      k_reconstruct<double, false, 0><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, nullptr, dt, flag);
-    else if (kind == 1)
-      k_reconstruct<double, false, 1><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, nullptr, dt, flag);
-    else
-      k_reconstruct<double, false, 2><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, nullptr, dt, flag);
-  }
+  const dim3 gs(blocks_for(g.P, 32), sh->ng ? 2 : 1);
+  const bool shared = recon_shared(sh, grid.x), mixed = sh->d.precision == CFFYN_MIXED;
+  if (!mixed) uf = nullptr;
+#define CFFYN_RECON_KIND(T_, K_)                                                                                      \
+  (shared ? (void)(k_reconstruct_shared<T_, K_><<<gs, 32 * kShares, 0, st>>>(sp, dst, g, mode, u, U, kacc, uf, dt,    \
+                                                                             flag))                                   \
+          : (void)(k_reconstruct<T_, false, K_><<<grid, 128, 0, st>>>(sp, dst, g, mode, u, U, kacc, uf, dt, flag)))
+  if (mixed)
+    kind == 0 ? CFFYN_RECON_KIND(ff, 0) : kind == 1 ? CFFYN_RECON_KIND(ff, 1) : CFFYN_RECON_KIND(ff, 2);
+  else
+    kind == 0 ? CFFYN_RECON_KIND(double, 0) : kind == 1 ? CFFYN_RECON_KIND(double, 1) : CFFYN_RECON_KIND(double, 2);
+#undef CFFYN_RECON_KIND
   count_launch();
   CF_CUDA(cudaGetLastError());
   return CFFYN_OK;

@@ -397,6 +397,376 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
   }
 }
 
+// k_rhs_gamma and k_rhs_quad for few points (rhs_shared): 32 points per block and
+// four warps, each warp a share of every point's tensors.  One thread's chain
+// through a whole point takes 30 and 25 us however few points there are; shared
+// out it takes 11 and 10 (13 x 9 x 18), at the price of barriers and repeated
+// 3+1 quantities.  The tensors live in shared memory as [slot][point], written by
+// one warp and read by all.  Every sum runs in the order of the kernels above:
+// the results are bit-identical.
+template <class T>
+struct PointSlots {
+  T* s;  // this point's column
+  __device__ __forceinline__ T& operator()(int v) const { return s[v * 32]; }
+};
+
+// slots of k_rhs_gamma_shared: g^ab, beta^i, alpha, n^a, Pi, Phi_iab, d_t g_ab,
+// Gamma_cab, C_a
+constexpr int kGG4 = 0, kGBu = 10, kGAl = 13, kGNu = 14, kGPi = 18, kGPh = 28, kGDt = 58, kGGam = 68, kGC = 108,
+              kGSlots = 112;
+
+// Warp 0 forms the 3+1 quantities while the others fetch Pi and Phi; the warps
+// share d_t g by component, Gamma_cab by c and the sources by b >= a.
+template <class T, bool FU, bool FO>
+__global__ void __launch_bounds__(kRhsBlock)
+    k_rhs_gamma_shared(const double* __restrict__ u, const double* __restrict__ H, const double* __restrict__ dH,
+                       double* __restrict__ src, double* __restrict__ out, Geo geo, int dtH) {
+  __shared__ T sm[kGSlots * 32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const PointSlots<T> V{sm + lane};
+  const long long P = geo.P;
+  const long long q = blockIdx.x * 32ll + lane;
+  const bool live = q < P;
+  const long long p = live ? q : P - 1;  // the last block's spare threads follow its last point
+  const T zero = S<T>::c(0.0), half = S<T>::c(0.5);
+
+  if (w == 0) {
+    T g[10];
+#pragma unroll
+    for (int s = 0; s < 10; ++s) g[s] = ldA<T, FU>(u, P, p, s);
+    Metric<T> M;
+    metric_from(g, M);
+#pragma unroll
+    for (int s = 0; s < 10; ++s) V(kGG4 + s) = M.gi4[s];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) V(kGBu + x) = M.bu[x];
+    V(kGAl) = M.alpha;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) V(kGNu + c) = M.nu[c];
+    if (live) {
+      stA<T, kInt<T>>(src, P, p, 40, M.alpha);
+#pragma unroll
+      for (int x = 0; x < 3; ++x) stA<T, kInt<T>>(src, P, p, 41 + x, M.bu[x]);
+      stA<T, kInt<T>>(src, P, p, 44, M.gi[0][0]);
+      stA<T, kInt<T>>(src, P, p, 45, M.gi[0][1]);
+      stA<T, kInt<T>>(src, P, p, 46, M.gi[0][2]);
+      stA<T, kInt<T>>(src, P, p, 47, M.gi[1][1]);
+      stA<T, kInt<T>>(src, P, p, 48, M.gi[1][2]);
+      stA<T, kInt<T>>(src, P, p, 49, M.gi[2][2]);
+    }
+  } else {
+    T v[14];
+#pragma unroll
+    for (int s = 0; s < 10; ++s) v[s] = ldA<T, FU>(u, P, p, 10 + 10 * w + s);  // Phi_iab, i = w - 1
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (w - 1 + 3 * s < 10) v[10 + s] = ldA<T, FU>(u, P, p, 10 + w - 1 + 3 * s);
+#pragma unroll
+    for (int s = 0; s < 10; ++s) V(kGPh + 10 * (w - 1) + s) = v[s];
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (w - 1 + 3 * s < 10) V(kGPi + w - 1 + 3 * s) = v[10 + s];
+  }
+  // H_a for every warp, d_a H_b for the warp's sources: in flight over the barrier
+  T Hd[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) Hd[a] = ldA<T, kInt<T>>(H, P, p, a);
+  __syncthreads();
+  const T alpha = V(kGAl);
+  // d_t g_ab (eq. gdot)
+#pragma unroll 1
+  for (int s = w; s < 10; s += 4) {
+    Acc<T> a;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) a.fma_(V(kGBu + x), V(kGPh + 10 * x + s));
+    a.fma_(-alpha, V(kGPi + s));
+    const T d = a.get();
+    V(kGDt + s) = d;
+    if (live) stA<T, FO>(out, P, p, s, d);
+  }
+  T gi4[10];
+#pragma unroll
+  for (int s = 0; s < 10; ++s) gi4[s] = V(kGG4 + s);
+  __syncthreads();
+  // Christoffel symbols Gamma_cab, c = w; Gamma_c = g^ab Gamma_cab (symmetric pairs
+  // counted twice off the diagonal) and the gauge constraint C_c = H_c + Gamma_c
+  {
+    const int c = w;
+    auto dg4 = [&](int e, int s) -> T { return V((e == 0 ? kGDt : kGPh + 10 * (e - 1)) + s); };
+    Acc<T> acc;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = a; b < 4; ++b) {
+        const T G = half * (dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
+        V(kGGam + c * 10 + SI(a, b)) = G;
+        const T wt = (a == b) ? gi4[SI(a, b)] : gi4[SI(a, b)] + gi4[SI(a, b)];
+        acc.fma_(wt, G);
+      }
+    acc.add(c == 0 ? Hd[0] : (c == 1 ? Hd[1] : (c == 2 ? Hd[2] : Hd[3])));
+    V(kGC + c) = acc.get();
+  }
+  __syncthreads();
+  // H^c, n^c C_c
+  T Hup[4], nC;
+  {
+    Acc<T> an;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      Acc<T> acc;
+#pragma unroll
+      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], Hd[d]);
+      Hup[c] = acc.get();
+      an.fma_(V(kGNu + c), V(kGC + c));
+    }
+    nC = an.get();
+  }
+  // the sources with larger index b = w
+  const int b = w;
+  T Gce[10];  // Gamma_b^{ce}, symmetric, off-diagonal weight 2
+  {
+    T Gcf[4][4];  // Gamma_b^c_f = g^cd Gamma_bdf
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        Acc<T> acc;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kGGam + b * 10 + SI(d, f)));
+        Gcf[c][f] = acc.get();
+      }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int e = c; e < 4; ++e) {
+        Acc<T> acc;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc.fma_(gi4[SI(e, f)], Gcf[c][f]);
+        Gce[SI(c, e)] = (c == e) ? acc.get() : acc.get() + acc.get();
+      }
+  }
+  const T twoal = alpha + alpha, m2al = -twoal;
+  const T aa = alpha * (-alpha);  // alpha n_0, n_a = (-alpha, 0, 0, 0)
+  const T anC = alpha * nC;
+#pragma unroll 1
+  for (int a = 0; a <= b; ++a) {
+    const int s = SI(a, b);
+    // S_Pi = -2 alpha nabla_(a H_b) + alpha (n_b C_a + n_a C_b - g_ab n^c C_c);
+    // d_a H_b: rows (x, b) = 4 x + b of dH for a = x + 1; d_t H_b is row 12 + b
+    // when the gauge source is evolved with its time derivative (58 fields),
+    // else zero
+    const T dHab = a == 0 ? (dtH ? ldA<T, kInt<T>>(dH, P, p, 12 + b) : zero)
+                          : ldA<T, kInt<T>>(dH, P, p, (a - 1) * 4 + b);
+    const T dHba = b == 0 ? (dtH ? ldA<T, kInt<T>>(dH, P, p, 12 + a) : zero)
+                          : ldA<T, kInt<T>>(dH, P, p, (b - 1) * 4 + a);
+    const T gab = ldA<T, FU>(u, P, p, s);
+    Acc<T> acc;
+    acc.fma_(half, dHab + dHba);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc.fma_(-V(kGGam + c * 10 + s), Hup[c]);
+    const T DH = acc.get();
+    Acc<T> v;
+    v.fma_(-twoal, DH);
+    v.fma_(-(anC), gab);
+    if (a == 0) v.fma_(aa, V(kGC + b));
+    if (b == 0) v.fma_(aa, V(kGC + a));
+    // -2 alpha g^cd g^ef Gamma_ace Gamma_bdf
+    Acc<T> qa;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int e = c; e < 4; ++e) qa.fma_(V(kGGam + a * 10 + SI(c, e)), Gce[SI(c, e)]);
+    Acc<T> r;
+    r.add(v.get());
+    r.fma_(m2al, qa.get());
+    if (live) stA<T, kInt<T>>(src, P, p, s, r.get());
+  }
+}
+
+// slots of k_rhs_quad_shared: Pi, Phi_iab, alpha | beta^i | gamma^ij as in the source
+// buffer
+constexpr int kQPi = 0, kQPh = 10, kQM = 40, kQSlots = 50;
+
+// Warp w takes the sources of d_t Pi_ab with larger index b = w and, w < 3, those
+// of d_t Phi_iab with i = w.
+template <class T, bool FU>
+__global__ void __launch_bounds__(kRhsBlock)
+    k_rhs_quad_shared(const double* __restrict__ u, double* __restrict__ src, Geo geo) {
+  __shared__ T sm[kQSlots * 32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const PointSlots<T> V{sm + lane};
+  const long long P = geo.P;
+  const long long q = blockIdx.x * 32ll + lane;
+  const bool live = q < P;
+  const long long p = live ? q : P - 1;
+  const T half = S<T>::c(0.5);
+  {
+    T v[13];
+#pragma unroll
+    for (int i = 0; i < 13; ++i) {
+      const int t = w + 4 * i;
+      if (t < 50) v[i] = t < 40 ? ldA<T, FU>(u, P, p, 10 + t) : ldA<T, kInt<T>>(src, P, p, t);
+    }
+#pragma unroll
+    for (int i = 0; i < 13; ++i) {
+      const int t = w + 4 * i;
+      if (t < 50) V(t) = v[i];
+    }
+  }
+  __syncthreads();
+  // 3+1 quantities (eqs. normal, abgfromgab) as k_rhs_gamma derived them
+  const T alpha = V(kQM);
+  T bu[3], gi[3][3];
+#pragma unroll
+  for (int x = 0; x < 3; ++x) bu[x] = V(kQM + 1 + x);
+  gi[0][0] = V(kQM + 4);
+  gi[0][1] = gi[1][0] = V(kQM + 5);
+  gi[0][2] = gi[2][0] = V(kQM + 6);
+  gi[1][1] = V(kQM + 7);
+  gi[1][2] = gi[2][1] = V(kQM + 8);
+  gi[2][2] = V(kQM + 9);
+  const T ialpha = S<T>::c(1.0) / alpha;
+  const T ia2 = ialpha * ialpha;
+  T nu[4];
+  nu[0] = ialpha;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) nu[i + 1] = -(bu[i] * ialpha);
+  const T hal = half * alpha;
+  {
+    T gi4[10];
+    gi4[0] = -ia2;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) gi4[SI(0, i + 1)] = bu[i] * ia2;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = i; j < 3; ++j) gi4[SI(i + 1, j + 1)] = gi[i][j] - bu[i] * bu[j] * ia2;
+    const T twoal = alpha + alpha;
+    const int b = w;
+    // Q2_ab = Pi_ac g^cd Pi_db, Q1_ab = gamma^ij g^cd Phi_iac Phi_jbd
+    T Piu[4], W[3][4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      Acc<T> acc;
+#pragma unroll
+      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kQPi + SI(b, d)));
+      Piu[c] = acc.get();
+    }
+    {
+      T Y[3][4];
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          Acc<T> acc;
+#pragma unroll
+          for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kQPh + 10 * x + SI(b, d)));
+          Y[x][c] = acc.get();
+        }
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          Acc<T> acc;
+#pragma unroll
+          for (int y = 0; y < 3; ++y) acc.fma_(gi[x][y], Y[y][c]);
+          W[x][c] = acc.get();
+        }
+    }
+    // remaining algebraic terms of eq. Pidot
+    T nnPi;
+    {
+      Acc<T> acc;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int d = 0; d < 4; ++d) acc.fma_(nu[c] * nu[d], V(kQPi + SI(c, d)));
+      nnPi = acc.get();
+    }
+    T cPh[3];  // beta^j - alpha n^c Pi_ci gamma^ij
+    {
+      T nPi[3];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        Acc<T> acc;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc.fma_(nu[c], V(kQPi + SI(c, x + 1)));
+        nPi[x] = acc.get();
+      }
+#pragma unroll
+      for (int y = 0; y < 3; ++y) {
+        Acc<T> acc;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) acc.fma_(nPi[x], gi[x][y]);
+        cPh[y] = bu[y] - alpha * acc.get();
+      }
+    }
+    const T cPi = -(hal * nnPi);
+#pragma unroll 1
+    for (int a = 0; a <= b; ++a) {
+      const int s = SI(a, b);
+      const T part = ldA<T, kInt<T>>(src, P, p, s);
+      Acc<T> q2;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) q2.fma_(-V(kQPi + SI(a, c)), Piu[c]);
+      Acc<T> qq;
+      qq.add(q2.get());
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) qq.fma_(V(kQPh + 10 * x + SI(a, c)), W[x][c]);
+      Acc<T> acc;
+      acc.add(part);
+      acc.fma_(twoal, qq.get());
+      acc.fma_(cPi, V(kQPi + s));
+#pragma unroll
+      for (int x = 0; x < 3; ++x) acc.fma_(cPh[x], V(kQPh + 10 * x + s));
+      if (live) stA<T, kInt<T>>(src, P, p, s, acc.get());
+    }
+  }
+  if (w == 3) return;
+  // algebraic terms of eq. Phidot
+  const int x = w;
+  T nnPhi;
+  {
+    Acc<T> acc;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int d = 0; d < 4; ++d) acc.fma_(nu[c] * nu[d], V(kQPh + 10 * x + SI(c, d)));
+    nnPhi = acc.get();
+  }
+  T Mk[3];  // alpha gamma^jk n^c Phi_x,j,c
+  {
+    T nP[3];
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+      Acc<T> acc;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc.fma_(nu[c], V(kQPh + 10 * x + SI(y + 1, c)));
+      nP[y] = acc.get();
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+      Acc<T> acc;
+#pragma unroll
+      for (int y = 0; y < 3; ++y) acc.fma_(nP[y], gi[y][z]);
+      Mk[z] = alpha * acc.get();
+    }
+  }
+  const T hnn = hal * nnPhi;
+#pragma unroll 1
+  for (int s = 0; s < 10; ++s) {
+    Acc<T> acc;
+    acc.fma_(hnn, V(kQPi + s));
+#pragma unroll
+    for (int z = 0; z < 3; ++z) acc.fma_(Mk[z], V(kQPh + 10 * z + s));
+    acc.fma_(-alpha, V(kQPh + 10 * x + s));
+    if (live) stA<T, kInt<T>>(src, P, p, 10 + 10 * x + s, acc.get());
+  }
+}
+
+// blockIdx.y: the block's share of the ten symmetric pairs (pp_split).
 template <class T, bool FO>
 __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, const double* __restrict__ src,
                                                 double* __restrict__ out, Geo geo) {
@@ -462,8 +832,9 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
       su[x] = acc.get();
     }
   }
+  const int per = 10 / (int)gridDim.y, s0 = per * (int)blockIdx.y;
 #pragma unroll 1
-  for (int s = 0; s < 10; ++s) {
+  for (int s = s0; s < s0 + per; ++s) {
     T Dd[3], DPh[3][3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
@@ -555,6 +926,27 @@ __global__ void __launch_bounds__(128) k_gauge_rhs(const double* __restrict__ u,
   }
 }
 
+// Whether a point's tensors are shared out over four warps: up to one wave of the
+// one-point-per-thread blocks (four per SM; gamma / quad, us, one thread against
+// four warps per point: 2106 points 30 / 25 against 11 / 10, 39168 points 37 / 38
+// against 29 / 35, 102400 points 69 / 72 against 69 / 74, 152064 points 81 / 91
+// against 97 / 106).
+// Blocks of a batch's other classes count too: beside them the shorter chain buys
+// nothing and the repeated work costs (batch of eight shells 14.7 against 15.4 ms).
+static bool rhs_shared(const cffyn_shell* sh, unsigned nbr) {
+  return nbr + sh->beside / kRhsBlock <= 4ll * sh->sm_count;
+}
+
+// Shares of the ten symmetric pairs per point in k_rhs_pp: one thread's loop over
+// all ten takes 27 us by itself (its loads wait one after the other), in ten
+// shares 9.5 (13 x 9 x 18); every share repeats the chain-rule coefficients, so
+// only as many are taken as fill one wave (four blocks per SM).
+static unsigned pp_split(const cffyn_shell* sh, unsigned nb) {
+  for (unsigned n : {10u, 5u, 2u})
+    if (nb * n + sh->beside / 128 <= 4ll * sh->sm_count) return n;
+  return 1u;
+}
+
 // stage = 0: all three kernels; 1: sources with Christoffels; 2: quadratic
 // sources; 3: principal parts + boundary.  u_pairs: the state is a pair-stored
 // internal buffer (the stage states of the mixed path); out_pairs: the output
@@ -563,7 +955,8 @@ __global__ void __launch_bounds__(128) k_gauge_rhs(const double* __restrict__ u,
 int pw_rhs_part(const cffyn_shell* sh, const double* u, const double* D, double* out, int stage,
                 bool u_pairs, bool out_pairs, cudaStream_t st) {
   Geo g = geo_of(sh);
-  const unsigned nb = blocks_for(g.P, 128), nbr = blocks_for(g.P, kRhsBlock);
+  const unsigned nb = blocks_for(g.P, 128), nbr = blocks_for(g.P, kRhsBlock), nbs = blocks_for(g.P, 32);
+  const bool shared = rhs_shared(sh, nbr);
   const bool mixed = sh->d.precision == CFFYN_MIXED;
   if (mixed && u_pairs != out_pairs) {
     set_error("internal: right-hand side storage (state %d, output %d) not instantiated", (int)u_pairs,
@@ -581,30 +974,40 @@ int pw_rhs_part(const cffyn_shell* sh, const double* u, const double* D, double*
         k_gauge_rhs<ff, false, false><<<nb, 128, 0, st>>>(u, D, sh->H, sh->dH, out, g);
       count_launch();
     }
+#define CFFYN_GAMMA(...)                                                                                       \
+  (shared ? (void)(k_rhs_gamma_shared<__VA_ARGS__><<<nbs, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, \
+                                                                              g, dtH))                         \
+          : (void)(k_rhs_gamma<__VA_ARGS__><<<nbr, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, g, dtH)))
     if (!mixed)
-      k_rhs_gamma<double, false, false><<<nbr, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, g, dtH);
+      CFFYN_GAMMA(double, false, false);
     else if (u_pairs)
-      k_rhs_gamma<ff, true, true><<<nbr, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, g, dtH);
+      CFFYN_GAMMA(ff, true, true);
     else
-      k_rhs_gamma<ff, false, false><<<nbr, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, g, dtH);
+      CFFYN_GAMMA(ff, false, false);
+#undef CFFYN_GAMMA
     count_launch();
   }
   if (stage == 0 || stage == 2) {
+#define CFFYN_QUAD(...)                                                                          \
+  (shared ? (void)(k_rhs_quad_shared<__VA_ARGS__><<<nbs, kRhsBlock, 0, st>>>(u, sh->Rsrc, g))    \
+          : (void)(k_rhs_quad<__VA_ARGS__><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g)))
     if (!mixed)
-      k_rhs_quad<double, false><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
+      CFFYN_QUAD(double, false);
     else if (u_pairs)
-      k_rhs_quad<ff, true><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
+      CFFYN_QUAD(ff, true);
     else
-      k_rhs_quad<ff, false><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
+      CFFYN_QUAD(ff, false);
+#undef CFFYN_QUAD
     count_launch();
   }
   if (stage == 0 || stage == 3) {
+    const dim3 npp(nb, pp_split(sh, nb));
     if (!mixed)
-      k_rhs_pp<double, false><<<nb, 128, 0, st>>>(D, sh->Rsrc, out, g);
+      k_rhs_pp<double, false><<<npp, 128, 0, st>>>(D, sh->Rsrc, out, g);
     else if (out_pairs)
-      k_rhs_pp<ff, true><<<nb, 128, 0, st>>>(D, sh->Rsrc, out, g);
+      k_rhs_pp<ff, true><<<npp, 128, 0, st>>>(D, sh->Rsrc, out, g);
     else
-      k_rhs_pp<ff, false><<<nb, 128, 0, st>>>(D, sh->Rsrc, out, g);
+      k_rhs_pp<ff, false><<<npp, 128, 0, st>>>(D, sh->Rsrc, out, g);
     count_launch();
   }
   CF_CUDA(cudaGetLastError());
