@@ -46,6 +46,7 @@ void free_tc(TcOp&);
 // pointwise.cu
 int pw_rhs(const cffyn_shell*, const double*, const double*, double*, cudaStream_t);
 int pw_rhs_part(const cffyn_shell*, const double*, const double*, double*, int, bool, bool, cudaStream_t);
+bool pw_rhs_shared(const cffyn_shell*);
 int pw_decompose(const cffyn_shell*, const double*, double*, bool, cudaStream_t);
 int pw_reconstruct(const cffyn_shell*, const double*, double*, int, double*, double*, double*, double*,
                    double, int*, cudaStream_t);
@@ -606,7 +607,8 @@ static int filter_in_step(cffyn_shell* sh, double* spin, cudaStream_t st, Run&& 
 // read the stage state only) run on the shell's second stream beside the
 // d_theta + d_phi launch, which they share no buffer with, and join before
 // the principal parts; forked after d_r (forked at the start of the stage,
-// they held up the exponent scan and d_r: 3.233 vs 3.248 ms per step); not
+// they held up the exponent scan and d_r: 3.233 vs 3.248 ms per step), but at
+// the start for small shells, whose launches leave SMs idle; not
 // for the evolved gauge of 54/58 fields (k_gauge_rhs reads the derivatives)
 // nor under per-group timing.
 template <class Run>
@@ -618,16 +620,21 @@ static int stage_front(cffyn_shell* sh, double* u, int s, cudaStream_t st, Run&&
   const double* X = stage_state_of(sh, u, s);
   int rc;
   const bool fork = conc && sh->ng == 0 && sh->aux_stream;
+  const bool early = fork && pw_rhs_shared(sh);
   cudaStream_t sa = fork ? sh->aux_stream : st;
-  if ((rc = run(10, [&] { return op_prepare(sh, X, xp, nf, P, 0, st); }))) return rc;
-  if ((rc = run(0, [&] { return op_deriv_r(sh, X, sh->D, nf, xp, st); }))) return rc;
-  if (fork) {
+  auto algebraic = [&]() -> int {
+    int r;
     CF_CUDA(cudaEventRecord(sh->ev_fork, st));
     CF_CUDA(cudaStreamWaitEvent(sa, sh->ev_fork, 0));
-    if ((rc = run(2, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 1, xp, true, sa); }))) return rc;
-    if ((rc = run(3, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 2, xp, true, sa); }))) return rc;
+    if ((r = run(2, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 1, xp, true, sa); }))) return r;
+    if ((r = run(3, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 2, xp, true, sa); }))) return r;
     CF_CUDA(cudaEventRecord(sh->ev_join, sa));
-  }
+    return CFFYN_OK;
+  };
+  if (early && (rc = algebraic())) return rc;
+  if ((rc = run(10, [&] { return op_prepare(sh, X, xp, nf, P, 0, st); }))) return rc;
+  if ((rc = run(0, [&] { return op_deriv_r(sh, X, sh->D, nf, xp, st); }))) return rc;
+  if (fork && !early && (rc = algebraic())) return rc;
   if ((rc = run(1, [&] { return op_deriv_theta_phi(sh, X, sh->D + nvP, sh->D + 2 * nvP, nf, xp, st); })))
     return rc;
   if (fork) {
@@ -742,17 +749,27 @@ int enqueue_step_branch(cffyn_shell* sh, double* u, double dt, cudaStream_t st, 
 // The pieces of a step for nested shells (no trace marks): stage s's
 // derivatives and right-hand side into sh->S, its filter and update, and
 // the per-step filter after the last stage.
-int enqueue_stage_front(cffyn_shell* sh, double* u, int s, cudaStream_t st) {
+// beside: the points of the nest's other shells, whose pieces run beside.
+int enqueue_stage_front(cffyn_shell* sh, double* u, int s, cudaStream_t st, long long beside) {
   auto run = [](int, auto&& fn) -> int { return fn(); };
-  return stage_front(sh, u, s, st, run, true);
+  sh->beside = beside;
+  const int rc = stage_front(sh, u, s, st, run, true);
+  sh->beside = 0;
+  return rc;
 }
-int enqueue_stage_back(cffyn_shell* sh, double* u, double dt, int s, cudaStream_t st) {
+int enqueue_stage_back(cffyn_shell* sh, double* u, double dt, int s, cudaStream_t st, long long beside) {
   auto run = [](int, auto&& fn) -> int { return fn(); };
-  return stage_back(sh, u, dt, s, st, run, true);
+  sh->beside = beside;
+  const int rc = stage_back(sh, u, dt, s, st, run, true);
+  sh->beside = 0;
+  return rc;
 }
-int enqueue_step_tail(cffyn_shell* sh, double* u, cudaStream_t st) {
+int enqueue_step_tail(cffyn_shell* sh, double* u, cudaStream_t st, long long beside) {
   auto run = [](int, auto&& fn) -> int { return fn(); };
-  return step_tail(sh, u, st, run, true);
+  sh->beside = beside;
+  const int rc = step_tail(sh, u, st, run, true);
+  sh->beside = 0;
+  return rc;
 }
 const double* stage_state(const cffyn_shell* sh, const double* u, int s) { return stage_state_of(sh, u, s); }
 

@@ -73,7 +73,7 @@ struct cffyn_shell {
   int device = 0;
   int sm_count = 1;             // SMs of the device: CTAs of a persistent launch
   long long beside = 0;         // points advanced beside this handle's launches while they are captured
-                                // (the other classes of a batch); 0 otherwise
+                                // (the other classes of a batch, the other shells of a nest); 0 otherwise
 
   // grid (device)
   double *r = nullptr, *sth = nullptr, *cth = nullptr, *sph = nullptr, *cph = nullptr;

@@ -30,9 +30,9 @@
 #include "pw_common.cuh"
 
 namespace cffyn {
-int enqueue_stage_front(cffyn_shell*, double*, int, cudaStream_t);
-int enqueue_stage_back(cffyn_shell*, double*, double, int, cudaStream_t);
-int enqueue_step_tail(cffyn_shell*, double*, cudaStream_t);
+int enqueue_stage_front(cffyn_shell*, double*, int, cudaStream_t, long long);
+int enqueue_stage_back(cffyn_shell*, double*, double, int, cudaStream_t, long long);
+int enqueue_step_tail(cffyn_shell*, double*, cudaStream_t, long long);
 int enqueue_step_prologue(cffyn_shell*, double*, cudaStream_t);
 int enqueue_rhs(cffyn_shell*, const double*, double*, cudaStream_t);
 const double* stage_state(const cffyn_shell*, const double*, int);
@@ -148,6 +148,10 @@ struct cffyn_nest {
   int device = 0;
   std::vector<cffyn_shell*> sh;
   cudaStream_t cap = nullptr;
+  // capture streams and join events of the shells' branches (shell 0: cap itself)
+  std::vector<cudaStream_t> br;
+  std::vector<cudaEvent_t> join;
+  cudaEvent_t fork = nullptr;
   cudaGraphExec_t graph = nullptr;
   std::vector<double*> gu;
   double gdt = 0.0;
@@ -163,27 +167,55 @@ void free_nest(cffyn_nest* ns) {
   cudaDeviceSynchronize();
   if (ns->graph) cudaGraphExecDestroy(ns->graph);
   if (ns->cap) cudaStreamDestroy(ns->cap);
+  for (cudaStream_t s : ns->br)
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t e : ns->join)
+    if (e) cudaEventDestroy(e);
+  if (ns->fork) cudaEventDestroy(ns->fork);
   if (ns->flags_host) cudaFreeHost(ns->flags_host);
   delete ns;
 }
 
-// One RK4 step of every shell of the nest on st.
+// fn(i, stream, points of the other shells) for every shell, as branches beside
+// one another forked from and joined into st (shell 0 on st itself): between two
+// couplings the shells share nothing, and a small shell's launches leave most of
+// the device idle.
+template <class F>
+int per_shell(cffyn_nest* ns, cudaStream_t st, F&& fn) {
+  long long all = 0;
+  for (const cffyn_shell* s : ns->sh) all += (long long)s->P;
+  int rc;
+  CF_CUDA(cudaEventRecord(ns->fork, st));
+  for (int i = ns->n - 1; i >= 0; --i) {
+    cudaStream_t b = i ? ns->br[i] : st;
+    if (i) CF_CUDA(cudaStreamWaitEvent(b, ns->fork, 0));
+    if ((rc = fn(i, b, all - (long long)ns->sh[i]->P))) return rc;
+    if (i) CF_CUDA(cudaEventRecord(ns->join[i], b));
+  }
+  for (int i = 1; i < ns->n; ++i) CF_CUDA(cudaStreamWaitEvent(st, ns->join[i], 0));
+  return CFFYN_OK;
+}
+
+// One RK4 step of every shell of the nest on st (a capture).
 int enqueue_nest_step(cffyn_nest* ns, double* const* u, double dt, cudaStream_t st) {
   int rc;
   const bool mixed = ns->sh[0]->d.precision == CFFYN_MIXED;
   for (int s = 0; s < 4; ++s) {
-    for (int i = 0; i < ns->n; ++i)
-      if ((rc = enqueue_stage_front(ns->sh[i], u[i], s, st))) return rc;
+    if ((rc = per_shell(ns, st, [&](int i, cudaStream_t b, long long beside) {
+           return enqueue_stage_front(ns->sh[i], u[i], s, b, beside);
+         })))
+      return rc;
     for (int i = 0; i + 1 < ns->n; ++i) {
       cffyn_shell* a = ns->sh[i];
       if ((rc = couple(a, ns->sh[i + 1], stage_state(a, u[i], s), a->S, ns->sh[i + 1]->S, mixed, mixed, st)))
         return rc;
     }
-    for (int i = 0; i < ns->n; ++i)
-      if ((rc = enqueue_stage_back(ns->sh[i], u[i], dt, s, st))) return rc;
+    if ((rc = per_shell(ns, st, [&](int i, cudaStream_t b, long long beside) {
+           const int r = enqueue_stage_back(ns->sh[i], u[i], dt, s, b, beside);
+           return r || s < 3 ? r : enqueue_step_tail(ns->sh[i], u[i], b, beside);
+         })))
+      return rc;
   }
-  for (int i = 0; i < ns->n; ++i)
-    if ((rc = enqueue_step_tail(ns->sh[i], u[i], st))) return rc;
   return CFFYN_OK;
 }
 
@@ -255,8 +287,17 @@ int cffyn_create_nest(int n, cffyn_shell* const* shells, cffyn_nest** out) {
   ns->dt_default = shells[0]->dt_default;
   for (int i = 1; i < n; ++i) ns->dt_default = std::min(ns->dt_default, shells[i]->dt_default);
   cudaError_t e;
+  ns->br.assign(n, nullptr);
+  ns->join.assign(n, nullptr);
+  auto branches = [&]() -> cudaError_t {
+    cudaError_t r = cudaEventCreateWithFlags(&ns->fork, cudaEventDisableTiming);
+    for (int i = 1; i < n && r == cudaSuccess; ++i)
+      if ((r = cudaStreamCreateWithFlags(&ns->br[i], cudaStreamNonBlocking)) == cudaSuccess)
+        r = cudaEventCreateWithFlags(&ns->join[i], cudaEventDisableTiming);
+    return r;
+  };
   if ((e = cudaStreamCreateWithFlags(&ns->cap, cudaStreamNonBlocking)) != cudaSuccess ||
-      (e = cudaMallocHost(&ns->flags_host, (size_t)n * sizeof(int))) != cudaSuccess) {
+      (e = branches()) != cudaSuccess || (e = cudaMallocHost(&ns->flags_host, (size_t)n * sizeof(int))) != cudaSuccess) {
     cudaGetLastError();
     set_error("nest creation: %s", cudaGetErrorString(e));
     free_nest(ns);

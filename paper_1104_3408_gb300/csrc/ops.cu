@@ -359,6 +359,12 @@ __device__ __forceinline__ unsigned int mag_key(long long w) {
 }
 
 template <bool FI>
+__device__ __forceinline__ int exp_word(unsigned int m) {
+  const int e = FI ? (int)(m >> 23) : (int)(m >> 20);
+  return FI ? (e ? e - 126 + 1022 : 0) : e;
+}
+
+template <bool FI>
 __global__ void __launch_bounds__(kExpThreads) k_field_exp(const long long* __restrict__ in, long long len,
                                                            int* __restrict__ exps) {
   __shared__ unsigned int wm[kExpThreads / 32];
@@ -388,9 +394,33 @@ __global__ void __launch_bounds__(kExpThreads) k_field_exp(const long long* __re
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < kExpThreads / 32; ++w) m = max(m, wm[w]);
-    const int e = FI ? (int)(m >> 23) : (int)(m >> 20);
-    const int word = FI ? (e ? e - 126 + 1022 : 0) : e;
+    const int word = exp_word<FI>(m);
     if (word) atomicMax(exps + f, word);
+  }
+}
+
+// The same for short fields, one CTA per field: the word is stored, so that the
+// words need no clearing in front (a launch less: 1.5 us of the 4.5 that the pair
+// takes on a 13 x 9 x 18 shell).
+constexpr int kExpShortThreads = 512, kExpShortLen = 16 * kExpShortThreads;
+
+template <bool FI>
+__global__ void __launch_bounds__(kExpShortThreads) k_field_exp_short(const long long* __restrict__ in, long long len,
+                                                                      int* __restrict__ exps) {
+  __shared__ unsigned int wm[kExpShortThreads / 32];
+  const long long* x = in + (long long)blockIdx.x * len;
+  unsigned int m = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int e = i * kExpShortThreads + threadIdx.x;
+    if (e < len) m = max(m, mag_key<FI>(__ldg(x + e)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = __reduce_max_sync(0xffffffffu, threadIdx.x < kExpShortThreads / 32 ? wm[threadIdx.x] : 0u);
+    if (threadIdx.x == 0) exps[blockIdx.x] = exp_word<FI>(m);
   }
 }
 
@@ -1335,10 +1365,22 @@ int set_op_smem_limits() {
 }
 
 // Per-field exponents of nf fields of len values each into exps (max(nf, 64)
-// words, zeroed here: they are atomicMax targets); in_pairs: pair-stored input.
-static int field_exps(const double* in, bool in_pairs, int nf, long long len, int* exps, cudaStream_t st) {
-  CF_CUDA(cudaMemsetAsync(exps, 0, sizeof(int) * std::max(nf, 64), st));
+// words; clear: also the words from nf on, which a caller uses, are zeroed);
+// in_pairs: pair-stored input.
+static int field_exps(const double* in, bool in_pairs, int nf, long long len, int* exps, cudaStream_t st,
+                      bool clear = false) {
   const long long* x = reinterpret_cast<const long long*>(in);
+  if (len <= kExpShortLen && !clear) {
+    if (in_pairs)
+      k_field_exp_short<true><<<nf, kExpShortThreads, 0, st>>>(x, len, exps);
+    else
+      k_field_exp_short<false><<<nf, kExpShortThreads, 0, st>>>(x, len, exps);
+    count_launch();
+    CF_CUDA(cudaGetLastError());
+    return CFFYN_OK;
+  }
+  // the words are atomicMax targets
+  CF_CUDA(cudaMemsetAsync(exps, 0, sizeof(int) * std::max(nf, 64), st));
   const unsigned bx = (unsigned)((len + kExpThreads * kExpPerThread - 1) / (kExpThreads * kExpPerThread));
   if (in_pairs)
     k_field_exp<true><<<dim3(bx, nf), kExpThreads, 0, st>>>(x, len, exps);
@@ -1612,7 +1654,7 @@ int op_derivs_at(const cffyn_shell* sh, const double* u, double* D, int nf, int*
   const long long P = (long long)sh->P;
   const bool mixed = sh->d.precision == CFFYN_MIXED;
   int rc;
-  if (mixed && (rc = field_exps(u, false, nf, P, exps, st))) return rc;
+  if (mixed && (rc = field_exps(u, false, nf, P, exps, st, true))) return rc;
   const double* W64[3] = {sh->Dr, sh->Dth2, sh->Dph};
   const TcOp* Wt[3] = {&sh->tDr, &sh->tDth2, &sh->tDph};
   for (int i = 0; i < 3; ++i)

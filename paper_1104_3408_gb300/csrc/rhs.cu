@@ -936,6 +936,7 @@ __global__ void __launch_bounds__(128) k_gauge_rhs(const double* __restrict__ u,
 static bool rhs_shared(const cffyn_shell* sh, unsigned nbr) {
   return nbr + sh->beside / kRhsBlock <= 4ll * sh->sm_count;
 }
+bool pw_rhs_shared(const cffyn_shell* sh) { return rhs_shared(sh, blocks_for((long long)P_all(sh), kRhsBlock)); }
 
 // Shares of the ten symmetric pairs per point in k_rhs_pp: one thread's loop over
 // all ten takes 27 us by itself (its loads wait one after the other), in ten

@@ -1,8 +1,9 @@
 """The persistent form of the split-precision operator kernel, which launches of
 many tiles take: derivatives and filter at shapes whose launches lie on both
 sides of its rule, with ragged tiles, both row-group sizes, the staged radial
-epilogue with 48 and 96 rows and the unstaged one (n_r > 80), against the plain
-FP64 operators.
+epilogue with 48 and 96 rows and the unstaged one (n_r > 80), and at the longest
+field of the one-block exponent scan (16 x 16 x 32) and the next above, against
+the plain FP64 operators.
 
 Tolerance of the derivatives: the 47-bit fixed point.  Column values are off by
 at most 2^-48 2^E <= 2^-47 max|u| and a row's entries by 2^-47 max|W|, so an
@@ -40,6 +41,7 @@ def _deriv_bound(sh, N, r_in, umax):
 
 @pytest.mark.parametrize("n_r,N,fields,rows", [
     (17, 32, 50, 0), (33, 47, 58, 0), (33, 47, 50, 48), (65, 24, 54, 0), (90, 16, 50, 0), (25, 48, 50, 96),
+    (16, 16, 50, 0), (17, 16, 58, 0),
 ])
 def test_persistent_launches_match_fp64(cf, n_r, N, fields, rows):
     u = torch.from_numpy(inputs.band_limited_fields(n_r, N, 2 * N, n_fields=fields, seed=n_r, bumps=2)).cuda()
