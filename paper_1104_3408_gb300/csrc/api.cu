@@ -29,8 +29,6 @@ void set_error(const char* fmt, ...) {
 // ops.cu
 int set_op_smem_limits();
 int op_deriv_r(const cffyn_shell*, const double*, double*, int, bool, cudaStream_t);
-int op_deriv_theta(const cffyn_shell*, const double*, double*, int, bool, cudaStream_t);
-int op_deriv_phi(const cffyn_shell*, const double*, double*, int, bool, cudaStream_t);
 int op_deriv_theta_phi(const cffyn_shell*, const double*, double*, double*, int, bool, cudaStream_t);
 int op_dft_fwd(const cffyn_shell*, const double*, double*, int, cudaStream_t, int, int f0 = 0);
 int op_dft_inv(const cffyn_shell*, const double*, double*, int, cudaStream_t, int, int, int f0 = 0);
@@ -51,7 +49,7 @@ int pw_decompose(const cffyn_shell*, const double*, double*, bool, cudaStream_t)
 int pw_reconstruct(const cffyn_shell*, const double*, double*, int, double*, double*, double*, double*,
                    double, int*, cudaStream_t);
 int pw_cart(const cffyn_shell*, const double*, double*, int, bool, cudaStream_t);
-int pw_triad_table(const cffyn_shell*);
+int pw_tables(const cffyn_shell*);
 int pw_gauge(const cffyn_shell*, const double*, double*, cudaStream_t);
 int pw_gauge_into_state(const cffyn_shell*, double*, cudaStream_t);
 int pw_to_internal(const cffyn_shell*, const double*, double*, long long, cudaStream_t);
@@ -133,9 +131,7 @@ int derivs_spherical(cffyn_shell* sh, const double* u, double* D, int nf, bool i
   int rc;
   if ((rc = op_prepare(sh, u, in_pairs, nf, (long long)P, 0, st))) return rc;
   if ((rc = op_deriv_r(sh, u, D, nf, in_pairs, st))) return rc;
-  if ((rc = op_deriv_theta(sh, u, D + (size_t)nf * P, nf, in_pairs, st))) return rc;
-  if ((rc = op_deriv_phi(sh, u, D + (size_t)2 * nf * P, nf, in_pairs, st))) return rc;
-  return CFFYN_OK;
+  return op_deriv_theta_phi(sh, u, D + (size_t)nf * P, D + (size_t)2 * nf * P, nf, in_pairs, st);
 }
 
 // Filter of the functions in `spin` (nv x P), in place, scratch D (2 nv P):
@@ -168,7 +164,7 @@ void free_shell(cffyn_shell* sh) {
   cudaDeviceSynchronize();
   double** ptrs[] = {&sh->r,   &sh->sth, &sh->cth,  &sh->sph,  &sh->cph,    &sh->Dr,     &sh->Dth2,
                      &sh->Dph, &sh->Fan, &sh->Fsy,  &sh->Fraw, &sh->Fproj0, &sh->FprojC, &sh->F0g, &sh->H,
-                     &sh->dH,  &sh->red, &sh->triad};
+                     &sh->dH,  &sh->red, &sh->triad, &sh->jinv, &sh->jinv_int, &sh->trig_int};
   for (double** p : ptrs)
     if (*p) cudaFree(*p);
   if (sh->ws_owned && sh->ws) cudaFree(sh->ws);
@@ -307,10 +303,14 @@ static int create_shell(const cffyn_shell_desc* desc, int ns, cffyn_shell** out)
     return CFFYN_OK;
   };
   if ((rc = alloc(&sh->H, 4 * P_all(sh))) || (rc = alloc(&sh->dH, (sh->nv == 58 ? 16 : 12) * P_all(sh))) ||
-      (rc = alloc(&sh->red, 2)) || (rc = alloc(&sh->triad, (size_t)9 * sh->N * sh->J)))
+      (rc = alloc(&sh->red, 2)) || (rc = alloc(&sh->triad, (size_t)9 * sh->N * sh->J)) ||
+      (rc = alloc(&sh->jinv, (size_t)2 * sh->N * sh->n_r)))
+    return fail(rc);
+  if (d.precision == CFFYN_MIXED && ((rc = alloc(&sh->jinv_int, (size_t)2 * sh->N * sh->n_r)) ||
+                                     (rc = alloc(&sh->trig_int, (size_t)2 * (sh->N + sh->J)))))
     return fail(rc);
   (void)nvP;
-  if ((rc = pw_triad_table(sh))) return fail(rc);
+  if ((rc = pw_tables(sh))) return fail(rc);
   if (d.precision == CFFYN_MIXED && cudaMalloc(&sh->exps, std::max(64, nv_ops(sh)) * sizeof(int)) != cudaSuccess)
     return fail(CFFYN_ENOMEM);
   sh->ws_bytes = ws_total_bytes(sh);

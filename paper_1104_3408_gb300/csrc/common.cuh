@@ -78,6 +78,10 @@ struct cffyn_shell {
   // grid (device)
   double *r = nullptr, *sth = nullptr, *cth = nullptr, *sph = nullptr, *cph = nullptr;
   double* triad = nullptr;  // [n_phi][n_theta][9] real triad rows, internal storage
+  // chain-rule factors 1 / r and 1 / (r sin theta), [n_theta][n_r][2], in FP64 and in
+  // internal storage, and the trigonometric factors sin, cos theta | sin, cos phi
+  // (2 n_theta, 2 n_phi) in internal storage
+  double *jinv = nullptr, *jinv_int = nullptr, *trig_int = nullptr;
 
   // FP64 operators (device, row-major)
   double* Dr = nullptr;     // n_r x n_r

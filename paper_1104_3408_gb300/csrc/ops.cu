@@ -1446,12 +1446,12 @@ int op_deriv_r(const cffyn_shell* sh, const double* in, double* out, int nfields
   return launch(sh, deriv_args(sh, 0, in, out, nfields), sh->Dr, &sh->tDr, dim3(1, 1), st, 0, in_pairs);
 }
 
-int op_deriv_theta(const cffyn_shell* sh, const double* in, double* out, int nfields, bool in_pairs,
+static int op_deriv_theta(const cffyn_shell* sh, const double* in, double* out, int nfields, bool in_pairs,
                    cudaStream_t st) {
   return launch(sh, deriv_args(sh, 1, in, out, nfields), sh->Dth2, &sh->tDth2, dim3(1, 1), st, 0, in_pairs);
 }
 
-int op_deriv_phi(const cffyn_shell* sh, const double* in, double* out, int nfields, bool in_pairs,
+static int op_deriv_phi(const cffyn_shell* sh, const double* in, double* out, int nfields, bool in_pairs,
                  cudaStream_t st) {
   return launch(sh, deriv_args(sh, 2, in, out, nfields), sh->Dph, &sh->tDph, dim3(1, 1), st, 0, in_pairs);
 }

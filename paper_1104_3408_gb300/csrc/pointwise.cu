@@ -19,6 +19,7 @@
 //   k_gauge        H_a = -Gamma_a (eq. gauge).
 //   k_constraints  sums of squares of C_iab = d_i g_ab - Phi_iab and
 //                  C_a = H_a + Gamma_a (App. A.1).
+#include <algorithm>
 #include <cstdio>
 #include <type_traits>
 
@@ -485,9 +486,8 @@ __global__ void __launch_bounds__(128) k_decompose(const double* __restrict__ in
   __shared__ T sm[kDecSlots * 128];
   const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (p >= geo.P) return;
-  const int i = (int)((p / geo.n_r) % geo.N);
-  const int jj = (int)((p / ((long long)geo.n_r * geo.N)) % geo.J);
-  const Triad<T> t = triad_at<T>(geo, i, jj);
+  const PointIdx x = point_idx(geo, p);
+  const Triad<T> t = triad_at<T>(geo, x.i, x.jj);
   decompose_group<T, FI>(group_of((int)blockIdx.y, (geo.nv - 50) / 4), Scratch<T>{sm}, in, out, geo.P, p, t);
 }
 
@@ -550,9 +550,8 @@ __device__ __forceinline__ void reconstruct_update(Scratch<T> sc, const double* 
     }
   };
   if (mode <= 4) {
-    const int i = (int)((p / geo.n_r) % geo.N);
-    const int jj = (int)((p / ((long long)geo.n_r * geo.N)) % geo.J);
-    const Triad<T> t = triad_at<T>(geo, i, jj);
+    const PointIdx x = point_idx(geo, p);
+    const Triad<T> t = triad_at<T>(geo, x.i, x.jj);
     reconstruct_group<T>(G, sc, sp, P, p, t, update);
   } else {
 #pragma unroll
@@ -779,9 +778,8 @@ __global__ void __launch_bounds__(32 * kShares, 4)
   StageUpdate<T, KIND> up{dst,   u,     U,     kacc,  uf, geo.P, x.p,
                           stage, x.live, false, S<T>::c(stage == 2 ? dt : 0.5 * dt), S<T>::c(dt / 6.0)};
   if (mode <= 4) {
-    const int i = (int)((x.p / geo.n_r) % geo.N);
-    const int jj = (int)((x.p / ((long long)geo.n_r * geo.N)) % geo.J);
-    const Triad<T> t = triad_at<T>(geo, i, jj);
+    const PointIdx at = point_idx(geo, x.p);
+    const Triad<T> t = triad_at<T>(geo, at.i, at.jj);
     auto emit = [&](int f, T k) { up.put(f, k, up.fetch(f)); };
     auto group = [&](int g) { reconstruct_group<T>(g, Scratch<T>{nullptr}, sp, geo.P, x.p, t, emit); };
     switch (x.share) {
@@ -834,27 +832,31 @@ __global__ void __launch_bounds__(32 * kShares, 4)
 
 // Spherical -> Cartesian derivatives: D[3][nf][P] -> out[3][nf][P] (FP64
 // arithmetic; D and out in the given storages).  Setup and API paths only.
-// One thread per point: the Jacobian (FP64 divisions) is formed once and
-// applied to every field, whose values are coalesced across the threads.
+// One thread per point and share of the fields (blockIdx.y, cart_split): the
+// Jacobian is formed once from the tables and applied to every field of the
+// share, whose values are coalesced across the threads.  Bound by the FP64 pipe
+// (eight operations per value at 0.49 T/s: 55 us for 50 fields of 33 x 32 x 64);
+// with all fields in one thread and the divisions in the kernel 118 us.
 // status (may be NULL): a status word of the operator launches that produced
 // D; if it is non-zero (a timed-out wait) every output value is a NaN.
 template <bool FI, bool FO>
-__global__ void k_cart(const double* __restrict__ D, double* __restrict__ out, int nf, Geo geo,
-                       const int* __restrict__ status) {
+__global__ void __launch_bounds__(256) k_cart(const double* __restrict__ D, double* __restrict__ out, int nf, Geo geo,
+                                              const int* __restrict__ status) {
   const long long P = geo.P;
   const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (p >= P) return;
+  const int per = (nf + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int mu0 = per * (int)blockIdx.y, mu1 = min(nf, mu0 + per);
   if (status && *status) {
     const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-    for (int e = 0; e < 3 * nf; ++e) Store<double, FO>::st(out, (long long)e * P + p, qnan);
+    for (int mu = mu0; mu < mu1; ++mu)
+      for (int x = 0; x < 3; ++x) Store<double, FO>::st(out, ((long long)x * nf + mu) * P + p, qnan);
     return;
   }
-  const int k = (int)(p % geo.n_r);
-  const int i = (int)((p / geo.n_r) % geo.N);
-  const int jj = (int)((p / ((long long)geo.n_r * geo.N)) % geo.J);
-  const Jac<double> J = jacobian<double>(geo, k, i, jj);
+  const PointIdx at = point_idx(geo, p);
+  const Jac<double> J = jacobian<double>(geo, at.k, at.i, at.jj);
 #pragma unroll 2
-  for (int mu = 0; mu < nf; ++mu) {
+  for (int mu = mu0; mu < mu1; ++mu) {
     const double dr = Store<double, FI>::ld(D, (long long)mu * P + p);
     const double dt = Store<double, FI>::ld(D, ((long long)nf + mu) * P + p);
     const double dp = Store<double, FI>::ld(D, ((long long)2 * nf + mu) * P + p);
@@ -862,6 +864,26 @@ __global__ void k_cart(const double* __restrict__ D, double* __restrict__ out, i
     for (int x = 0; x < 3; ++x)
       Store<double, FO>::st(out, ((long long)x * nf + mu) * P + p,
                             J.j[x][0] * dr + J.j[x][1] * dt + J.j[x][2] * dp);
+  }
+}
+
+// Tables of the chain rule's factors (see cffyn_shell), formed in T arithmetic.
+template <class T, bool F>
+__global__ void k_jac_tables(Geo g, double* jinv, double* trig) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < g.N * g.n_r) {
+    const int i = e / g.n_r, k = e - i * g.n_r;
+    const T ir = S<T>::c(1.0) / S<T>::c(g.r[k]);
+    Store<T, F>::st(jinv, 2 * (long long)e, ir);
+    Store<T, F>::st(jinv, 2 * (long long)e + 1, ir / S<T>::c(g.sth[i]));
+  }
+  if (trig && e < g.N) {
+    Store<T, F>::st(trig, e, S<T>::c(g.sth[e]));
+    Store<T, F>::st(trig, g.N + e, S<T>::c(g.cth[e]));
+  }
+  if (trig && e < g.J) {
+    Store<T, F>::st(trig, 2 * g.N + e, S<T>::c(g.sph[e]));
+    Store<T, F>::st(trig, 2 * g.N + g.J + e, S<T>::c(g.cph[e]));
   }
 }
 
@@ -992,12 +1014,18 @@ int pw_reconstruct(const cffyn_shell* sh, const double* sp, double* dst, int mod
   return CFFYN_OK;
 }
 
+// Shares of nf fields in k_cart: about eight blocks per SM.
+static dim3 cart_grid(const cffyn_shell* sh, const Geo& g, int nf) {
+  const unsigned nb = blocks_for(g.P, 256), want = (8u * (unsigned)sh->sm_count + nb - 1) / nb;
+  return dim3(nb, std::max(1u, std::min(want, (unsigned)(nf + 4) / 5)));
+}
+
 // D: internal storage; out_pairs: out is an internal buffer; status: see k_cart
 int pw_cart_status(const cffyn_shell* sh, const double* D, double* out, int nf, bool out_pairs,
                    const int* status, cudaStream_t st) {
   Geo g = geo_of(sh);
   const bool in_pairs = sh->d.precision == CFFYN_MIXED;
-  const unsigned nb = blocks_for(g.P, 256);
+  const dim3 nb = cart_grid(sh, g, nf);
   if (in_pairs && out_pairs)
     k_cart<true, true><<<nb, 256, 0, st>>>(D, out, nf, g, status);
   else if (in_pairs)
@@ -1017,15 +1045,19 @@ int pw_cart(const cffyn_shell* sh, const double* D, double* out, int nf, bool ou
 // on either path (the FFT derivative path writes FP64 into the workspace)
 int pw_cart_fp64(const cffyn_shell* sh, const double* D, double* out, int nf, cudaStream_t st) {
   Geo g = geo_of(sh);
-  k_cart<false, false><<<blocks_for(g.P, 256), 256, 0, st>>>(D, out, nf, g, nullptr);
+  k_cart<false, false><<<cart_grid(sh, g, nf), 256, 0, st>>>(D, out, nf, g, nullptr);
   count_launch();
   CF_CUDA(cudaGetLastError());
   return CFFYN_OK;
 }
 
-// Table of the real triad rows at every (theta_i, phi_j) (set-up).
-int pw_triad_table(const cffyn_shell* sh) {
+// Tables of the real triad rows at every (theta_i, phi_j) and of the chain
+// rule's factors (set-up).
+int pw_tables(const cffyn_shell* sh) {
   Geo g = geo_of(sh);
+  const unsigned nj = blocks_for(std::max((long long)g.N * g.n_r, (long long)g.J), 128);
+  k_jac_tables<double, false><<<nj, 128>>>(g, sh->jinv, nullptr);
+  if (sh->d.precision == CFFYN_MIXED) k_jac_tables<ff, true><<<nj, 128>>>(g, sh->jinv_int, sh->trig_int);
   const unsigned nb = blocks_for((long long)g.N * g.J, 128);
   if (sh->d.precision == CFFYN_MIXED)
     k_triad_table<ff><<<nb, 128>>>(g, sh->triad);

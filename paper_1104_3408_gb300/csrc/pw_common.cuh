@@ -12,6 +12,7 @@ struct Geo {
   long long P;
   const double *r, *sth, *cth, *sph, *cph;
   const double* triad;  // [J][N][9] rows of the real triad (internal storage)
+  const double *jinv, *jinv_int, *trig_int;  // see cffyn_shell
 };
 
 // symmetric pair index of (a, b), a, b in 0..3 (tt,tx,ty,tz,xx,xy,xz,yy,yz,zz)
@@ -29,14 +30,44 @@ struct Jac {
   T st, ct, sp, cp;
 };
 
+// The factors of a point's Jacobian: 1 / r, 1 / (r sin theta), sin and cos of theta
+// and phi.  Read from tables of the set-up (the divisions and, in double-float,
+// the conversions cost as much as two components' derivatives).
+template <class T>
+struct JacFactors {
+  T ir, irs, st, ct, sp, cp;
+};
+template <class T>
+__device__ __forceinline__ JacFactors<T> jac_factors(const Geo& g, int k, int i, int jj);
+template <>
+__device__ __forceinline__ JacFactors<double> jac_factors<double>(const Geo& g, int k, int i, int jj) {
+  const double2 v = __ldg(reinterpret_cast<const double2*>(g.jinv) + i * g.n_r + k);
+  return {v.x, v.y, g.sth[i], g.cth[i], g.sph[jj], g.cph[jj]};
+}
+template <>
+__device__ __forceinline__ JacFactors<ff> jac_factors<ff>(const Geo& g, int k, int i, int jj) {
+  using L = Store<ff, true>;
+  const long long o = 2 * ((long long)i * g.n_r + k);
+  const double* t = g.trig_int;
+  return {L::ld(g.jinv_int, o), L::ld(g.jinv_int, o + 1), L::ld(t, i), L::ld(t, g.N + i), L::ld(t, 2 * g.N + jj),
+          L::ld(t, 2 * g.N + g.J + jj)};
+}
+
+// radial, polar and azimuthal index of point p (of the point within its shell
+// for stacked shells; points are fewer than 2^31)
+struct PointIdx {
+  int k, i, jj;
+};
+__device__ __forceinline__ PointIdx point_idx(const Geo& g, long long p) {
+  const unsigned q = (unsigned)p / (unsigned)g.n_r, j = q / (unsigned)g.N;
+  return {(int)((unsigned)p - q * (unsigned)g.n_r), (int)(q - j * (unsigned)g.N), (int)(j % (unsigned)g.J)};
+}
+
 template <class T>
 __device__ __forceinline__ Jac<T> jacobian(const Geo& g, int k, int i, int jj) {
   Jac<T> J;
-  const T st = S<T>::c(g.sth[i]), ct = S<T>::c(g.cth[i]);
-  const T sp = S<T>::c(g.sph[jj]), cp = S<T>::c(g.cph[jj]);
-  const T one = S<T>::c(1.0);
-  const T ir = one / S<T>::c(g.r[k]);
-  const T irs = ir / st;
+  const JacFactors<T> f = jac_factors<T>(g, k, i, jj);
+  const T st = f.st, ct = f.ct, sp = f.sp, cp = f.cp, ir = f.ir, irs = f.irs;
   J.j[0][0] = st * cp; J.j[0][1] = ct * cp * ir; J.j[0][2] = -(sp * irs);
   J.j[1][0] = st * sp; J.j[1][1] = ct * sp * ir; J.j[1][2] = cp * irs;
   J.j[2][0] = ct;      J.j[2][1] = -(st * ir);   J.j[2][2] = S<T>::c(0.0);
@@ -136,6 +167,9 @@ inline Geo geo_of(const cffyn_shell* sh) {
   g.sph = sh->sph;
   g.cph = sh->cph;
   g.triad = sh->triad;
+  g.jinv = sh->jinv;
+  g.jinv_int = sh->jinv_int;
+  g.trig_int = sh->trig_int;
   return g;
 }
 

@@ -63,6 +63,15 @@ __device__ __forceinline__ float u64_scaled_to_float(unsigned long long v, int s
   return __uint_as_float(bits);
 }
 
+// The same of a 32-bit integer.
+__device__ __forceinline__ float u32_scaled_to_float(unsigned int v, int sc, bool neg) {
+  const int nb = 32 - __clz((int)v);
+  const int ex = nb + 126 + sc;  // biased
+  const unsigned int m = nb > 24 ? v >> (nb - 24) : v << (24 - nb);
+  if (v == 0 || ex <= 0) return 0.0f;  // zero, or below the normal range: flushed
+  return __uint_as_float((neg ? 0x80000000u : 0u) | ((unsigned int)ex << 23) | (m & 0x7fffffu));
+}
+
 // Split an FP64 value into hi + lo with integer operations only: hi keeps the
 // leading 24 significand bits (truncated), lo the next 24 (truncated), so
 // |x - hi - lo| <= 2^-47 |x|.  Values outside the FP32 normal range are
@@ -76,18 +85,29 @@ __device__ __forceinline__ ff ff_from_double(double x) {
   const int E = e - 1023;
   if (E > 127) return ff{neg ? -__int_as_float(0x7f800000) : __int_as_float(0x7f800000), 0.0f};
   if (E < -126) return ff{0.0f, 0.0f};
-  const unsigned long long m = b & 0x000fffffffffffffull;
-  const unsigned int hbits = (neg ? 0x80000000u : 0u) | ((unsigned int)(E + 127) << 23) |
-                             (unsigned int)(m >> 29);
-  const float hi = __uint_as_float(hbits);
-  const float lo = u64_scaled_to_float(m & ((1ull << 29) - 1), E - 52, neg);
-  return ff{hi, lo};
+  const unsigned int bh = (unsigned int)(b >> 32), bl = (unsigned int)b;
+  const unsigned int hbits = (bh & 0x80000000u) | ((unsigned int)(E + 127) << 23) |
+                             (__funnelshift_l(bl, bh, 3) & 0x7fffffu);
+  return ff{__uint_as_float(hbits), u32_scaled_to_float(bl & 0x1fffffffu, E - 52, neg)};
 }
 
 // hi + lo as a double with integer operations only.
 __device__ __forceinline__ double ff_to_double(ff a) {
   const unsigned int uh = __float_as_uint(a.hi), ul = __float_as_uint(a.lo);
   const int eh = (int)((uh >> 23) & 0xff), el = (int)((ul >> 23) & 0xff);
+  if ((unsigned int)(eh - 1) < 254u && eh - el >= 24) {
+    // a normalised pair (|lo| at most half an ulp of hi): the sum V of the two
+    // significands in units of 2^(eh - 127 - 52) has 53 bits, or 52 when lo takes
+    // hi below a power of two
+    const unsigned int Ml = el ? (ul & 0x7fffffu) | 0x800000u : 0u;
+    const int sh = el - eh + 29;  // at most 5
+    const unsigned int Lv = sh >= 0 ? Ml << sh : (sh > -32 ? Ml >> -sh : 0u);
+    const unsigned long long Mh = (unsigned long long)((uh & 0x7fffffu) | 0x800000u) << 29;
+    const unsigned long long V = ((uh ^ ul) >> 31) ? Mh - Lv : Mh + Lv;
+    const int below = (int)(V >> 52) ^ 1;
+    const unsigned long long bits = ((unsigned long long)(unsigned int)(eh + 895 - below) << 52) + (V << below);
+    return __longlong_as_double((long long)(bits | ((unsigned long long)(uh >> 31) << 63)));
+  }
   if (eh == 0xff) return (double)a.hi;         // Inf / NaN
   if (eh == 0) {                                // hi zero (or FP32 denormal): lo alone
     if (el == 0) return 0.0;
