@@ -768,16 +768,49 @@ __global__ void __launch_bounds__(kRhsBlock)
   }
 }
 
+// Asynchronous copy of one 8-byte word to shared memory (the thread's own word:
+// it waits for its own copies, no barrier).
+__device__ __forceinline__ void copy8_async(void* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned int)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+template <int N>
+__device__ __forceinline__ void copies_pending_at_most() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// The words of a symmetric pair (15 derivatives, 4 sources) are copied to shared
+// memory one pair ahead: held in registers only one pair's loads were in flight
+// (DRAM 54 %, half the warps' time waiting for them).
+constexpr int kPpWords = 19;
+
 // blockIdx.y: the block's share of the ten symmetric pairs (pp_split).
 template <class T, bool FO>
 __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, const double* __restrict__ src,
                                                 double* __restrict__ out, Geo geo) {
+  __shared__ T buf[2][kPpWords][128];
   const long long P = geo.P;
   const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (p >= P) return;
   const PointIdx at = point_idx(geo, p);
   const int k = at.k, i = at.i, jj = at.jj;
   const int nv = geo.nv;
+  const int per = 10 / (int)gridDim.y, s0 = per * (int)blockIdx.y;
+  // words 5 m .. 5 m + 4: d_m of g_s, Pi_s, Phi_xs; 15: source of d_t Pi_s, 16..18:
+  // of d_t Phi_xs
+  auto fetch = [&](int s) {
+    T(*w)[128] = buf[(s - s0) & 1];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const double* d = D + (long long)m * nv * P + p;
+#pragma unroll
+      for (int e = 0; e < 5; ++e) copy8_async(&w[5 * m + e][threadIdx.x], d + (long long)(10 * e + s) * P);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) copy8_async(&w[15 + e][threadIdx.x], src + (long long)(10 * e + s) * P + p);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(s0);
   const T half = S<T>::c(0.5);
   const Jac<T> J = jacobian<T>(geo, k, i, jj);
   const T alpha = ldA<T, kInt<T>>(src, P, p, 40);
@@ -833,21 +866,24 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
       su[x] = acc.get();
     }
   }
-  const int per = 10 / (int)gridDim.y, s0 = per * (int)blockIdx.y;
 #pragma unroll 1
   for (int s = s0; s < s0 + per; ++s) {
+    if (s + 1 < s0 + per) {
+      fetch(s + 1);
+      copies_pending_at_most<1>();
+    } else {
+      copies_pending_at_most<0>();
+    }
+    auto word = [&](int e) -> T { return buf[(s - s0) & 1][e][threadIdx.x]; };
     T Dd[3], DPh[3][3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      const long long base = (long long)m * nv * P + p;
-      const T dg = Store<T, kInt<T>>::ld(D, base + (long long)s * P);
-      const T dpi = Store<T, kInt<T>>::ld(D, base + (long long)(10 + s) * P);
-      Dd[m] = dg - dpi;
+      Dd[m] = word(5 * m) - word(5 * m + 1);
 #pragma unroll
-      for (int x = 0; x < 3; ++x) DPh[x][m] = Store<T, kInt<T>>::ld(D, base + (long long)(20 + 10 * x + s) * P);
+      for (int x = 0; x < 3; ++x) DPh[x][m] = word(5 * m + 2 + x);
     }
     Acc<T> aPi;
-    aPi.add(ldA<T, kInt<T>>(src, P, p, s));
+    aPi.add(word(15));
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       aPi.fma_(-b[m], Dd[m]);
@@ -859,7 +895,7 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
       Acc<T> a;
-      a.add(ldA<T, kInt<T>>(src, P, p, 10 + 10 * x + s));
+      a.add(word(16 + x));
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
         a.fma_(b[m], DPh[x][m]);
