@@ -495,7 +495,8 @@ struct TcBatch {
 // thread layout of a CTA
 constexpr int kEpiWarps = 8, kProdGroups = 3;
 constexpr int kProdWarp0 = kEpiWarps, kMmaWarp = kProdWarp0 + 4 * kProdGroups, kLoadWarp = kMmaWarp + 1;
-constexpr int kWsThreads = 32 * (kLoadWarp + 1);  // 704
+constexpr int kRawWarp = kLoadWarp + 1;               // d_r's input copies (STAGE 2)
+constexpr int kWsThreads = 32 * (kRawWarp + 1);  // 736
 
 template <int ROWS>
 struct WsCfg {
@@ -506,9 +507,8 @@ struct WsCfg {
   static constexpr uint32_t kTmemCols = 512;                           // set i at column 256 i
   static_assert(kStage % 1024 == 0, "stage alignment of the descriptors and bulk copies");
 };
-// stages of the ring; the staged epilogue of d_r takes one stage's room for
-// the outputs (see stage_bytes)
-template <int ROWS, bool STAGE>
+// stages of the ring; d_r's tiles (STAGE 1 and 2) take one stage's room and more
+template <int ROWS, int STAGE>
 constexpr int kRingStages = (ROWS == 48 ? 4 : 3) - (STAGE ? 1 : 0);
 constexpr int kTcMaxSmem = 224 * 1024;  // of 227 KB, beside the barriers and row factors
 
@@ -646,22 +646,33 @@ struct ColScale {
       : f1(f2_dup(pow2f(ec))), f2_(f2_dup(pow2f(ec - max(-126, min(127, ec))))), extreme(ec < -60 || ec > 60) {}
 };
 
-// The folded pairs of rows j and j + 1 of a chunk of accumulator rows v;
-// rowF: those rows' 2^E_row (8-byte aligned).
-template <int N>
-__device__ __forceinline__ void fold_rows(const uint32_t (&v)[5][N], int j, const float* rowF, const ColScale& cs,
-                                          long long& w0, long long& w1) {
-  auto two = [&](int d) { return f2_pack(__uint_as_float(v[d][j]), __uint_as_float(v[d][j + 1])); };
-  const float2 rr = *reinterpret_cast<const float2*>(rowF);
-  const f2 rf = f2_pack(rr.x, rr.y);
-  f2 hi, lo;
-  fold_pairs(two(0), two(1), two(2), two(3), two(4), cs.extreme ? rf : f2_mul(rf, cs.f1), hi, lo);
-  if (cs.extreme) {
-    hi = f2_mul(f2_mul(hi, cs.f1), cs.f2_);
-    lo = f2_mul(f2_mul(lo, cs.f1), cs.f2_);
+// The folded pairs w of a chunk of N accumulator rows v; rowF: those rows' 2^E_row
+// (8-byte aligned).
+template <bool EXTREME, int N>
+__device__ __forceinline__ void fold_rows(const uint32_t (&v)[5][N], const float* rowF, const ColScale& cs,
+                                          long long (&w)[N]) {
+#pragma unroll
+  for (int j = 0; j < N; j += 2) {
+    auto two = [&](int d) { return f2_pack(__uint_as_float(v[d][j]), __uint_as_float(v[d][j + 1])); };
+    const float2 rr = *reinterpret_cast<const float2*>(rowF + j);
+    const f2 rf = f2_pack(rr.x, rr.y);
+    f2 hi, lo;
+    fold_pairs(two(0), two(1), two(2), two(3), two(4), EXTREME ? rf : f2_mul(rf, cs.f1), hi, lo);
+    if (EXTREME) {
+      hi = f2_mul(f2_mul(hi, cs.f1), cs.f2_);
+      lo = f2_mul(f2_mul(lo, cs.f1), cs.f2_);
+    }
+    w[j] = (long long)((lo << 32) | f2_lo(hi));
+    w[j + 1] = (long long)((lo & 0xffffffff00000000ull) | f2_hi(hi));
   }
-  w0 = (long long)((lo << 32) | f2_lo(hi));
-  w1 = (long long)((lo & 0xffffffff00000000ull) | f2_hi(hi));
+}
+template <int N>
+__device__ __forceinline__ void fold_chunk(const uint32_t (&v)[5][N], const float* rowF, const ColScale& cs,
+                                           long long (&w)[N]) {
+  if (__any_sync(0xffffffffu, cs.extreme))
+    fold_rows<true>(v, rowF, cs, w);
+  else
+    fold_rows<false>(v, rowF, cs, w);
 }
 
 // Digit slices of two float pairs x = hi + lo (|lo| < ulp(hi), |x| < 2^E) on
@@ -732,16 +743,22 @@ __device__ __forceinline__ int col_exponent(const TcBatch& B, const OpArgs& a, c
   return ce - 1022 + B.eoff;
 }
 
-// STAGE: the launch is d_r (one operator class, all rows in one group): the
-// epilogue stages a tile's outputs in shared memory and stores them as one
-// contiguous block per 32 columns.
-template <bool FI, int ROWS, bool STAGE = false>
+// STAGE: the launch is d_r (one operator class, all rows in one group), whose
+// columns are contiguous lines of n_r words.  1: the epilogue stages a tile's
+// outputs in shared memory and stores them as one contiguous block per 32
+// columns.  2 (ROWS = 48, odd n_r up to kRawRows): also the inputs come as one bulk
+// copy per tile, into one of two buffers that the tile's outputs then take (each
+// thread's 16 words of a line, 8 bytes per load and a line apart across the
+// lanes, were 32 sectors per load: 61 against 38 us for 50 fields of 33 x 48 x 96;
+// odd, so that the lanes' words lie in different banks).
+constexpr int kRawRows = 39;
+template <bool FI, int ROWS, int STAGE>
 __global__ void __launch_bounds__(kWsThreads, 1)
     k_op_ws(const __grid_constant__ TcBatch B, const int* __restrict__ exps, int pairing, int* __restrict__ flag) {
   using C = WsCfg<ROWS>;
   constexpr int S = kRingStages<ROWS, STAGE>, A = C::kAccs;
   extern __shared__ __align__(1024) unsigned char smtc[];
-  __shared__ uint64_t xfull[S], wfull[S], empty[S], accfull[A], accempty[A], drained;
+  __shared__ uint64_t xfull[S], wfull[S], empty[S], accfull[A], accempty[A], rawfull[2], rawfree[2], drained;
   __shared__ uint32_t tmem_base;
   __shared__ __align__(16) float rowF[kEpiWarps][ROWS / 2];  // 2^E_row of each epilogue warp's rows
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -756,6 +773,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       tc::bar_init(&accfull[i], 1);
       tc::bar_init(&accempty[i], kEpiWarps);
     }
+    for (int i = 0; i < 2; ++i) {
+      tc::bar_init(&rawfull[i], 1);
+      tc::bar_init(&rawfree[i], kEpiWarps);
+    }
     tc::bar_init(&drained, 1);
   }
   if (warp == kMmaWarp) tc::alloc(&tmem_base, C::kTmemCols);
@@ -764,22 +785,27 @@ __global__ void __launch_bounds__(kWsThreads, 1)
   tc::fence_after();
   const uint32_t tm = tmem_base;
   bool ok = true;
+  // d_r's tile of item n of this CTA: [column][n_r]
+  auto tile_buf = [&](int n) {
+    return reinterpret_cast<long long*>(smtc + S * C::kStage) + (STAGE == 2 ? (n & 1) * kTcCols * B.a[0].g.P : 0);
+  };
 
   if (warp >= kProdWarp0 && warp < kMmaWarp) {
     // a group must not be two uses of a stage ahead of the products (its wait
     // on `empty` tells phases apart by their parity only): with two stages
     // the third group has no part
-    constexpr int G = S < kProdGroups ? S : kProdGroups;
+    // (for the same reason every group takes part in every tile of STAGE 2)
+    const int G = STAGE == 2 ? min(kProdGroups, B.W[0].ksteps) : (S < kProdGroups ? S : kProdGroups);
     const int g = (warp - kProdWarp0) >> 2;
     const int ctile = (warp & 3) * 32 + lane;
     const int xoff = (ctile >> 3) * 256 + (ctile & 7) * 16;
-    int t = blockIdx.x, ks = g;
+    int t = blockIdx.x, n = 0, ks = g;
     TcItem x;
     ColDesc col;
     int E = 0;
     // the group's next k-step: k-step ks of item t, or of a later item
     auto settle = [&](bool fresh) -> bool {
-      for (; t < total; t += gridDim.x) {
+      for (; t < total; t += gridDim.x, ++n) {
         if (fresh) x = item_at(B, t);
         if (ks < x.ksteps) {
           if (fresh) {
@@ -797,10 +823,17 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     };
     long long w[16];
     bool have = g < G && settle(true);
-    if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);
+    if (STAGE != 2 && have) gather16<FI>(B.a[x.cls], col, ks * 16, w);
     for (int it = g; have; it += G) {
       const int s = it % S, use = it / S;
       if (use > 0 && !(ok = __all_sync(0xffffffffu, pipe_wait(&empty[s], (use - 1) & 1, B.wait_ns)))) break;
+      if constexpr (STAGE == 2) {
+        if (!(ok = __all_sync(0xffffffffu, pipe_wait(&rawfull[n & 1], (n >> 1) & 1, B.wait_ns)))) break;
+        const int P = B.a[0].g.P;
+        const long long* line = tile_buf(n) + ctile * P;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = ks * 16 + i < P ? line[ks * 16 + i] : 0ll;
+      }
       unsigned char* xs = smtc + s * C::kStage + xoff;
       const bool fscale = FI && E >= -78 && E <= 126;  // FMA-pipe slicing of float pairs
       const f2 sc = f2_dup(pow2f(fscale ? 7 - E : 0)), sc3 = f2_dup(pow2f(fscale ? 31 - E : 0));
@@ -828,9 +861,26 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       bar_arrive(&xfull[s]);
       ks += G;
       have = settle(false);
-      if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);
+      if (STAGE != 2 && have) gather16<FI>(B.a[x.cls], col, ks * 16, w);
     }
   } else if (warp >= kMmaWarp) {
+    if (STAGE == 2 && warp == kRawWarp && lane == 0) {
+      int n = 0;
+      const int P = B.a[0].g.P;
+      for (int t = blockIdx.x; t < total; t += gridDim.x, ++n) {
+        if (n >= 2 && !(ok = pipe_wait(&rawfree[n & 1], ((n >> 1) - 1) & 1, B.wait_ns))) break;
+        const long long c0 = item_at(B, t).tile * kTcCols;
+        const int words = (int)min((long long)kTcCols, B.a[0].g.ncols - c0) * P;
+        const long long* src = reinterpret_cast<const long long*>(B.a[0].in) + c0 * P;
+        long long* dst = tile_buf(n);
+        // whole 16 bytes by the bulk copy, the odd last word of the last tile here
+        if (words & 1) dst[words - 1] = __ldg(src + words - 1);
+        const uint32_t bytes = (uint32_t)(words >> 1) * 16;
+        tc::bar_expect_tx(&rawfull[n & 1], bytes);
+        if (bytes) tc::bulk_g2s(dst, src, bytes, &rawfull[n & 1]);
+      }
+      for (int c = n > 2 ? n - 2 : 0; c < n; ++c) tc::bar_wait(&rawfull[c & 1], (c >> 1) & 1, kTcWaitNs);
+    }
     if (warp == kLoadWarp && lane == 0) {
       // the operator slices of a k-step; without the digit-sum-6 pairs the
       // last five (digits 1..5 times 2^-16) stay in global memory
@@ -930,7 +980,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       long long* o0 = out + col.out0;
       const long long ors = a.g.out_rs;
       long long* o1 = out + col.out1 - a.g.P0 * ors;
-      long long* stage = reinterpret_cast<long long*>(smtc + S * C::kStage) + (size_t)ctile * prow;
+      long long* stage = STAGE ? tile_buf(n) + ctile * prow : nullptr;
       if (h * R >= pend) {
         __syncwarp();
         if (lane == 0) bar_arrive(&accempty[ai]);
@@ -949,42 +999,54 @@ __global__ void __launch_bounds__(kWsThreads, 1)
           __syncwarp();
           if (lane == 0) bar_arrive(&accempty[ai]);
         }
+        long long w[CH];
+        fold_chunk(v, rf + p0 - h * R, cs, w);
         const int p = prow0 + p0;
-        const bool whole = p0 + CH <= pend && (p >= a.g.P0 || p + CH <= a.g.P0);
-        long long* o = (p >= a.g.P0 ? o1 : o0) + p * ors;  // a chunk within one output segment
+        if (STAGE) {
 #pragma unroll
-        for (int j = 0; j < CH; j += 2) {
-          long long w0, w1;
-          fold_rows(v, j, rf + p0 - h * R + j, cs, w0, w1);
-          if (STAGE) {
-            if (p0 + j < pend) stage[p0 + j] = w0;
-            if (p0 + j + 1 < pend) stage[p0 + j + 1] = w1;
-          } else if (whole) {
-            if (col.valid) {
-              *o = w0;
-              o += ors;
-              *o = w1;
-              o += ors;
-            }
-          } else if (col.valid) {
-            if (p0 + j < pend) (p + j >= a.g.P0 ? o1 : o0)[(p + j) * ors] = w0;
-            if (p0 + j + 1 < pend) (p + j + 1 >= a.g.P0 ? o1 : o0)[(p + j + 1) * ors] = w1;
+          for (int j = 0; j < CH; ++j)
+            if (p0 + j < pend) stage[p0 + j] = w[j];
+        } else if (p0 + CH <= pend && (p >= a.g.P0 || p + CH <= a.g.P0)) {
+          // a chunk within one output segment: one pointer and its stride
+          if (col.valid) {
+            long long* o = (p >= a.g.P0 ? o1 : o0) + p * ors;
+#pragma unroll
+            for (int j = 0; j < CH; ++j, o += ors) *o = w[j];
           }
+        } else if (col.valid) {
+#pragma unroll
+          for (int j = 0; j < CH; ++j)
+            if (p0 + j < pend) (p + j >= a.g.P0 ? o1 : o0)[(p + j) * ors] = w[j];
         }
       }
-      if constexpr (STAGE) {
+      if constexpr (STAGE != 0) {
         // d_r: a quarter's outputs (32 columns of n_r rows each, out0 = c n_r)
-        // are one contiguous block, copied out with consecutive threads on
-        // consecutive words
+        // are one contiguous block: a bulk store, or for the columns of the last
+        // tile consecutive threads on consecutive words
+        tc::fence_proxy_async();
         named_sync(1 + q, 64);
         const long long c0 = x.tile * kTcCols + q * 32;
         const int words = (int)max(0ll, min(32ll, a.g.ncols - c0)) * prow;
-        const long long* from = reinterpret_cast<const long long*>(smtc + S * C::kStage) + (size_t)q * 32 * prow;
+        const long long* from = tile_buf(n) + q * 32 * prow;
         long long* dst = out + c0 * prow;
-        for (int e = h * 32 + lane; e < words; e += 64) dst[e] = from[e];
-        named_sync(1 + q, 64);
+        if (words == 32 * prow) {
+          if (h == 0 && lane == 0) {
+            tc::bulk_s2g(dst, from, (uint32_t)words * 8);
+            tc::bulk_read_wait();
+          }
+        } else {
+          for (int e = h * 32 + lane; e < words; e += 64) dst[e] = from[e];
+          tc::fence_proxy_async();
+        }
+        if (STAGE == 1) {
+          named_sync(1 + q, 64);
+        } else {
+          __syncwarp();
+          if (lane == 0) bar_arrive(&rawfree[n & 1]);
+        }
       }
     }
+    if (STAGE && h == 0 && lane == 0) tc::bulk_done_wait();
   }
   ok = __syncthreads_and(ok);
   if (!ok && threadIdx.x == 0) atomicOr(flag, 2);
@@ -1226,13 +1288,11 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads)
         tc::ld_wait(v[0]);
 #pragma unroll
         for (int d = 1; d < 5; ++d) tc::tie(v[d]);
+        long long w[8];
+        fold_chunk(v, rowF + p0, cs, w);
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-          long long w0, w1;
-          fold_rows(v, j, rowF + p0 + j, cs, w0, w1);
-          if (p0 + j < prow) sink(p0 + j, w0);
-          if (p0 + j + 1 < prow) sink(p0 + j + 1, w1);
-        }
+        for (int j = 0; j < 8; ++j)
+          if (p0 + j < prow) sink(p0 + j, w[j]);
       }
     };
     if constexpr (!stage_out)
@@ -1295,28 +1355,34 @@ static int launch_batch(const cffyn_shell* sh, const TcBatch& b0, cudaStream_t s
   // d_r (one class, one row group): the instance with the staged epilogue
   const bool dr = b.nclass == 1 && b.a[0].kind == OP_R && b.W[0].ngroups == 1;
   const bool persistent = runs_persistent(sh, rows, items);
-#define CFFYN_LAUNCH_TC(R_, FI_, ST_)                                                                        \
-  (persistent ? (void)(k_op_ws<FI_, R_, ST_><<<sh->sm_count, kWsThreads,                                      \
-                                               kRingStages<R_, ST_> * WsCfg<R_>::kStage + (ST_ ? out_bytes : 0), \
-                                               st>>>(b, exps, pairing, flag))                                \
-              : (void)(k_op_tc<FI_, R_, ST_><<<(unsigned)items, TcCfg<R_>::kThreads, TcCfg<R_>::kSmem, st>>>( \
-                    b, exps, pairing, flag)))
-  // the persistent instance keeps the staged outputs beside its ring
-  const int out_bytes = kTcCols * b.a[0].g.P * (int)sizeof(double);
-  const int ring = rows == 48 ? WsCfg<48>::kStage * kRingStages<48, true> : WsCfg<96>::kStage * kRingStages<96, true>;
-  const bool stage = dr && (!persistent || ring + out_bytes <= kTcMaxSmem);
-  if (rows == 48) {
-    if (in_pairs)
-      stage ? CFFYN_LAUNCH_TC(48, true, true) : CFFYN_LAUNCH_TC(48, true, false);
-    else
-      stage ? CFFYN_LAUNCH_TC(48, false, true) : CFFYN_LAUNCH_TC(48, false, false);
+  const int P = b.a[0].g.P, out_bytes = kTcCols * P * (int)sizeof(double);
+  // d_r's tiles beside the persistent kernel's ring
+  const int ring = rows == 48 ? WsCfg<48>::kStage * kRingStages<48, 1> : WsCfg<96>::kStage * kRingStages<96, 1>;
+  const int stage = !dr || (persistent && ring + out_bytes > kTcMaxSmem) ? 0
+                    : persistent && rows == 48 && (P & 1) && P <= kRawRows ? 2
+                                                                           : 1;
+#define CFFYN_LAUNCH_WS(R_, FI_, ST_)                                                                        \
+  k_op_ws<FI_, R_, ST_><<<sh->sm_count, kWsThreads, kRingStages<R_, ST_> * WsCfg<R_>::kStage + ST_ * out_bytes, st>>>( \
+      b, exps, pairing, flag)
+#define CFFYN_LAUNCH_TC(R_, FI_, ST_) \
+  k_op_tc<FI_, R_, ST_><<<(unsigned)items, TcCfg<R_>::kThreads, TcCfg<R_>::kSmem, st>>>(b, exps, pairing, flag)
+#define CFFYN_LAUNCH_OP(FI_)                                                                                       \
+  if (!persistent && rows == 48)                                                                                   \
+    stage ? CFFYN_LAUNCH_TC(48, FI_, true) : CFFYN_LAUNCH_TC(48, FI_, false);                                      \
+  else if (!persistent)                                                                                            \
+    stage ? CFFYN_LAUNCH_TC(96, FI_, true) : CFFYN_LAUNCH_TC(96, FI_, false);                                      \
+  else if (rows == 48)                                                                                             \
+    stage == 0 ? CFFYN_LAUNCH_WS(48, FI_, 0) : stage == 1 ? CFFYN_LAUNCH_WS(48, FI_, 1) : CFFYN_LAUNCH_WS(48, FI_, 2); \
+  else                                                                                                             \
+    stage == 0 ? CFFYN_LAUNCH_WS(96, FI_, 0) : CFFYN_LAUNCH_WS(96, FI_, 1)
+  if (in_pairs) {
+    CFFYN_LAUNCH_OP(true);
   } else {
-    if (in_pairs)
-      stage ? CFFYN_LAUNCH_TC(96, true, true) : CFFYN_LAUNCH_TC(96, true, false);
-    else
-      stage ? CFFYN_LAUNCH_TC(96, false, true) : CFFYN_LAUNCH_TC(96, false, false);
+    CFFYN_LAUNCH_OP(false);
   }
+#undef CFFYN_LAUNCH_OP
 #undef CFFYN_LAUNCH_TC
+#undef CFFYN_LAUNCH_WS
   count_launch();
   CF_CUDA(cudaGetLastError());
   return CFFYN_OK;
@@ -1353,11 +1419,11 @@ static int launch(const cffyn_shell* sh, const OpArgs& a, const double* W64, con
 
 int set_op_smem_limits() {
   CF_CUDA(cudaFuncSetAttribute(k_op_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-#define CFFYN_TC_INSTANCES(k) \
-  (const void*)k<true, 48>, (const void*)k<false, 48>, (const void*)k<true, 96>, (const void*)k<false, 96>, \
-      (const void*)k<true, 48, true>, (const void*)k<false, 48, true>, (const void*)k<true, 96, true>, \
-      (const void*)k<false, 96, true>
-  const void* tcs[] = {CFFYN_TC_INSTANCES(k_op_ws), CFFYN_TC_INSTANCES(k_op_tc)};
+#define CFFYN_TC_INSTANCES(FI_)                                                                                   \
+  (const void*)k_op_tc<FI_, 48, false>, (const void*)k_op_tc<FI_, 48, true>, (const void*)k_op_tc<FI_, 96, false>, \
+      (const void*)k_op_tc<FI_, 96, true>, (const void*)k_op_ws<FI_, 48, 0>, (const void*)k_op_ws<FI_, 48, 1>,      \
+      (const void*)k_op_ws<FI_, 48, 2>, (const void*)k_op_ws<FI_, 96, 0>, (const void*)k_op_ws<FI_, 96, 1>
+  const void* tcs[] = {CFFYN_TC_INSTANCES(true), CFFYN_TC_INSTANCES(false)};
 #undef CFFYN_TC_INSTANCES
   for (const void* f : tcs)
     CF_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem));

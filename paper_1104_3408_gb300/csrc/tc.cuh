@@ -80,6 +80,17 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// Bulk store of `bytes` (multiple of 16; both addresses 16-byte aligned) from this
+// CTA's shared memory to global memory, as a bulk group of this thread.
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\ncp.async.bulk.commit_group;" ::"l"(dst),
+               "r"(smem_addr(src)), "r"(bytes)
+               : "memory");
+}
+// Waits until this thread's bulk stores have read their shared memory / are done.
+__device__ __forceinline__ void bulk_read_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_done_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 // TMEM allocation of ncols columns (power of two >= 32) by one whole warp; the
 // base address is written to *dst (shared memory).
 __device__ __forceinline__ void alloc(uint32_t* dst, uint32_t ncols) {

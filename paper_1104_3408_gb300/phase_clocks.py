@@ -33,9 +33,9 @@ NAMES = ["mma: wait for operator copies", "mma: wait for slices", "mma: wait for
 
 # (text of the kernel, text with the clocks) pairs applied to a copy of csrc/ops.cu
 _PATCHES = [
-    ("// STAGE: the launch is d_r (one operator class, all rows in one group): the",
+    ("// STAGE: the launch is d_r (one operator class, all rows in one group), whose",
      "__device__ unsigned long long g_instr[1024][16];\n#define CK clock64()\n"
-     "// STAGE: the launch is d_r (one operator class, all rows in one group): the"),
+     "// STAGE: the launch is d_r (one operator class, all rows in one group), whose"),
     ("  const int total = B.first[B.nclass];\n",
      "  const int total = B.first[B.nclass];\n  const long long c_entry = CK;\n  long long ins[12] = {0};\n"),
     ("  const uint32_t tm = tmem_base;\n", "  const uint32_t tm = tmem_base;\n  const long long c_setup = CK;\n"),
@@ -43,8 +43,8 @@ _PATCHES = [
     ("      unsigned char* xs = smtc + s * C::kStage + xoff;\n",
      "      unsigned char* xs = smtc + s * C::kStage + xoff;\n      const long long p1_ = CK;\n"),
     ("      bar_arrive(&xfull[s]);\n", "      bar_arrive(&xfull[s]);\n      const long long p2_ = CK;\n"),
-    ("      if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);\n    }\n",
-     "      if (have) gather16<FI>(B.a[x.cls], col, ks * 16, w);\n      ins[5] += p1_ - p0_;\n      ins[6] += p2_ - p1_;\n"
+    ("      if (STAGE != 2 && have) gather16<FI>(B.a[x.cls], col, ks * 16, w);\n    }\n",
+     "      if (STAGE != 2 && have) gather16<FI>(B.a[x.cls], col, ks * 16, w);\n      ins[5] += p1_ - p0_;\n      ins[6] += p2_ - p1_;\n"
      "      ins[7] += CK - p2_;\n    }\n"),
     ("        const int ai = n % A, ause = n / A;\n        if (ause > 0",
      "        const int ai = n % A, ause = n / A;\n        const long long a0_ = CK;\n        if (ause > 0"),
@@ -61,9 +61,9 @@ _PATCHES = [
      "      long long e1_ = CK, e2_ = 0;\n"),
     ("          // the accumulators are read: the next item may overwrite them\n",
      "          e2_ = CK;\n          // the accumulators are read: the next item may overwrite them\n"),
-    ("      if constexpr (STAGE) {\n        // d_r: a quarter",
+    ("      if constexpr (STAGE != 0) {\n        // d_r: a quarter",
      "      ins[8] += e1_ - e0_;\n      if (e2_) ins[9] += e2_ - e1_, ins[10] += CK - e2_;\n"
-     "      if constexpr (STAGE) {\n        // d_r: a quarter"),
+     "      if constexpr (STAGE != 0) {\n        // d_r: a quarter"),
     ("  ok = __syncthreads_and(ok);\n",
      "  if (!STAGE && B.sum6 && B.nclass == 2 && lane == 0) {\n    const int lo = warp == kMmaWarp ? 0 : warp == kProdWarp0 ? 5 : warp == 0 ? 8 : 12;\n"
      "    const int hi = warp == kMmaWarp ? 5 : warp == kProdWarp0 ? 8 : warp == 0 ? 11 : 12;\n"
