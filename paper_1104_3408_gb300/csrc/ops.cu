@@ -173,11 +173,17 @@ __device__ __forceinline__ void store_elem(const OpArgs& a, const ColDesc& d, in
 }
 
 // ---------------------------------------------------------------------------
-// FP64 core: CTA tile = PT rows x QT columns, whole K staged in shared memory.
+// FP64 core: CTA tile = 8 RP rows x QT columns, whole K staged in shared memory;
+// each of eight warps holds RP rows.  Bound by the FP64 pipe, which a row past
+// the operator's end costs as much as a row within (17 x 16 x 32, 64 rows for
+// every operator: d_r with 17 rows 64 us, d_theta with 32 rows 60 us), so the
+// rows are cut into as few equal tiles of at most 64 as there can be, rounded up
+// to eight.
 
 constexpr int F64_QT = 32;
-constexpr int F64_PT = 64;
+constexpr int F64_MAX_RP = 8;
 
+template <int RP>
 __global__ void __launch_bounds__(256) k_op_fp64(OpArgs a, const double* __restrict__ W) {
   extern __shared__ double sm64[];
   if (a.batched_m) {
@@ -185,10 +191,11 @@ __global__ void __launch_bounds__(256) k_op_fp64(OpArgs a, const double* __restr
     W += (size_t)a.m * a.w_stride;
   }
   const int K = a.g.K, P = a.g.P;
-  const int p0 = blockIdx.y * F64_PT;
-  const int PT = min(F64_PT, P - p0);
+  constexpr int TILE = 8 * RP;
+  const int p0 = blockIdx.y * TILE;
+  const int PT = min(TILE, P - p0);
   double* Ws = sm64;                 // PT x K
-  double* Xs = sm64 + F64_PT * K;    // K x QT
+  double* Xs = sm64 + TILE * K;      // K x QT
   __shared__ ColDesc cols[F64_QT];
   const long long c0 = (long long)blockIdx.x * F64_QT;
   const int tid = threadIdx.x;
@@ -203,23 +210,25 @@ __global__ void __launch_bounds__(256) k_op_fp64(OpArgs a, const double* __restr
   }
   __syncthreads();
   const int tq = tid % F64_QT, tp = tid / F64_QT;  // 8 row groups
-  double acc[F64_PT / 8];
+  double acc[RP];
+  const double* wrow[RP];
 #pragma unroll
-  for (int r = 0; r < F64_PT / 8; ++r) acc[r] = 0.0;
+  for (int r = 0; r < RP; ++r) {
+    acc[r] = 0.0;
+    wrow[r] = Ws + min(tp + 8 * r, PT - 1) * K;  // a row past the end repeats the last
+  }
+#pragma unroll 2
   for (int k = 0; k < K; ++k) {
-    double x = Xs[k * F64_QT + tq];
+    const double x = Xs[k * F64_QT + tq];
 #pragma unroll
-    for (int r = 0; r < F64_PT / 8; ++r) {
-      int row = tp + 8 * r;
-      if (row < PT) acc[r] = fma(Ws[row * K + k], x, acc[r]);
-    }
+    for (int r = 0; r < RP; ++r) acc[r] = fma(wrow[r][k], x, acc[r]);
   }
   if (kfast) {
     // transpose through shared memory so that stores run along p
     __syncthreads();
     double* Os = Xs;  // reuse: PT x QT
 #pragma unroll
-    for (int r = 0; r < F64_PT / 8; ++r) {
+    for (int r = 0; r < RP; ++r) {
       int row = tp + 8 * r;
       if (row < PT) Os[row * F64_QT + tq] = acc[r];
     }
@@ -230,7 +239,7 @@ __global__ void __launch_bounds__(256) k_op_fp64(OpArgs a, const double* __restr
     }
   } else {
 #pragma unroll
-    for (int r = 0; r < F64_PT / 8; ++r) {
+    for (int r = 0; r < RP; ++r) {
       int row = tp + 8 * r;
       if (row < PT) store_elem(a, cols[tq], p0 + row, acc[r]);
     }
@@ -1397,10 +1406,25 @@ static int launch(const cffyn_shell* sh, const OpArgs& a, const double* W64, con
                   int sum6 = 1, int* flag = nullptr) {
   if (a.g.ncols <= 0) return CFFYN_OK;
   if (sh->d.precision == CFFYN_FP64 || Wt == nullptr) {
-    unsigned gx = (unsigned)((a.g.ncols + F64_QT - 1) / F64_QT);
-    unsigned gy = (unsigned)((a.g.P + F64_PT - 1) / F64_PT);
-    size_t smem = (size_t)(F64_PT * a.g.K + a.g.K * F64_QT) * sizeof(double);
-    k_op_fp64<<<dim3(gx, gy, extra.y), 256, smem, st>>>(a, W64);
+    const unsigned gx = (unsigned)((a.g.ncols + F64_QT - 1) / F64_QT);
+    const int nt = (a.g.P + 8 * F64_MAX_RP - 1) / (8 * F64_MAX_RP);        // row tiles
+    const int rp = ((a.g.P + nt - 1) / nt + 7) / 8;                        // rows per warp
+    const unsigned gy = (unsigned)((a.g.P + 8 * rp - 1) / (8 * rp));
+    const size_t smem = (size_t)(8 * rp * a.g.K + a.g.K * F64_QT) * sizeof(double);
+    const dim3 grid(gx, gy, extra.y);
+    switch (rp) {
+#define CFFYN_FP64_CASE(RP_)                                 \
+  case RP_: k_op_fp64<RP_><<<grid, 256, smem, st>>>(a, W64); break;
+      CFFYN_FP64_CASE(1)
+      CFFYN_FP64_CASE(2)
+      CFFYN_FP64_CASE(3)
+      CFFYN_FP64_CASE(4)
+      CFFYN_FP64_CASE(5)
+      CFFYN_FP64_CASE(6)
+      CFFYN_FP64_CASE(7)
+      CFFYN_FP64_CASE(8)
+#undef CFFYN_FP64_CASE
+    }
     count_launch();
     CF_CUDA(cudaGetLastError());
     return CFFYN_OK;
@@ -1418,7 +1442,10 @@ static int launch(const cffyn_shell* sh, const OpArgs& a, const double* W64, con
 }
 
 int set_op_smem_limits() {
-  CF_CUDA(cudaFuncSetAttribute(k_op_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  const void* f64[] = {(const void*)k_op_fp64<1>, (const void*)k_op_fp64<2>, (const void*)k_op_fp64<3>,
+                       (const void*)k_op_fp64<4>, (const void*)k_op_fp64<5>, (const void*)k_op_fp64<6>,
+                       (const void*)k_op_fp64<7>, (const void*)k_op_fp64<8>};
+  for (const void* f : f64) CF_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
 #define CFFYN_TC_INSTANCES(FI_)                                                                                   \
   (const void*)k_op_tc<FI_, 48, false>, (const void*)k_op_tc<FI_, 48, true>, (const void*)k_op_tc<FI_, 96, false>, \
       (const void*)k_op_tc<FI_, 96, true>, (const void*)k_op_ws<FI_, 48, 0>, (const void*)k_op_ws<FI_, 48, 1>,      \
