@@ -194,7 +194,6 @@ template <class T, bool FI>
 __device__ __forceinline__ void decompose_group(int grp, Scratch<T> sc, const double* __restrict__ in,
                                                 double* __restrict__ out, long long P, long long p,
                                                 const Triad<T>& t) {
-  const T two = S<T>::c(2.0);
   switch (grp) {
     case 0:
       st<kIn<T>>(out, P, p, SLOT_R0(0), ld<T, FI>(in, P, p, SI(0, 0)));
@@ -230,7 +229,7 @@ __device__ __forceinline__ void decompose_group(int grp, Scratch<T> sc, const do
       st<kIn<T>>(out, P, p, SLOT_C1(3 + gph), O[0][1]);
       st<kIn<T>>(out, P, p, SLOT_C1(3 + gph) + 1, O[0][2]);
       st<kIn<T>>(out, P, p, SLOT_C2(gph), O[1][1] - O[2][2]);
-      st<kIn<T>>(out, P, p, SLOT_C2(gph) + 1, two * O[1][2]);
+      st<kIn<T>>(out, P, p, SLOT_C2(gph) + 1, twice(O[1][2]));
       break;
     }
     case 6: {
@@ -287,7 +286,7 @@ __device__ __forceinline__ void decompose_group(int grp, Scratch<T> sc, const do
         T O[6];
 #pragma unroll
         for (int q = 0; q < 6; ++q) O[q] = r0 * sc(q) + r1 * sc(6 + q) + r2 * sc(12 + q);
-        const T pr = O[0], pmb = O[3] + O[5], prm0 = O[1], prm1 = O[2], pmm0 = O[3] - O[5], pmm1 = two * O[4];
+        const T pr = O[0], pmb = O[3] + O[5], prm0 = O[1], prm1 = O[2], pmm0 = O[3] - O[5], pmm1 = twice(O[4]);
         if (A == 0) {
           st<kIn<T>>(out, P, p, SLOT_R0(10), pr);
           st<kIn<T>>(out, P, p, SLOT_R0(11), pmb);
@@ -327,7 +326,6 @@ __device__ __forceinline__ void decompose_group(int grp, Scratch<T> sc, const do
 template <class T, class Emit>
 __device__ __forceinline__ void reconstruct_group(int grp, Scratch<T> sc, const double* __restrict__ sp, long long P,
                                                   long long p, const Triad<T>& t, Emit&& emit) {
-  const T half = S<T>::c(0.5);
   switch (grp) {
     case 0:
       emit(SI(0, 0), ld<T, kIn<T>>(sp, P, p, SLOT_R0(0)));
@@ -359,9 +357,9 @@ __device__ __forceinline__ void reconstruct_group(int grp, Scratch<T> sc, const 
       O[0][0] = rr;
       O[0][1] = O[1][0] = rmr;
       O[0][2] = O[2][0] = rmi;
-      O[1][1] = half * (mmb + mmr);
-      O[2][2] = half * (mmb - mmr);
-      O[1][2] = O[2][1] = half * mmi;
+      O[1][1] = half_of(mmb + mmr);
+      O[2][2] = half_of(mmb - mmr);
+      O[1][2] = O[2][1] = half_of(mmi);
       unrot_mat(t, O, Tm);
 #pragma unroll
       for (int a = 0; a < 3; ++a)
@@ -379,10 +377,10 @@ __device__ __forceinline__ void reconstruct_group(int grp, Scratch<T> sc, const 
       O[0][2] = ld<T, kIn<T>>(sp, P, p, SLOT_C1(5) + 1);
       O[1][0] = ld<T, kIn<T>>(sp, P, p, SLOT_C1(6));
       O[2][0] = ld<T, kIn<T>>(sp, P, p, SLOT_C1(6) + 1);
-      O[1][1] = half * (s42 + s12);
-      O[2][2] = half * (s12 - s42);
-      O[1][2] = half * (s43 - s13);
-      O[2][1] = half * (s43 + s13);
+      O[1][1] = half_of(s42 + s12);
+      O[2][2] = half_of(s12 - s42);
+      O[1][2] = half_of(s43 - s13);
+      O[2][1] = half_of(s43 + s13);
       unrot_mat(t, O, Tm);
 #pragma unroll
       for (int a = 0; a < 3; ++a)
@@ -418,19 +416,19 @@ __device__ __forceinline__ void reconstruct_group(int grp, Scratch<T> sc, const 
         // X = (m; rm) = P^th + i P^ph, Y = (m; r mbar) = conj(P^th) + i conj(P^ph)
         const T xr = ld<T, kIn<T>>(sp, P, p, SLOT_C2(4)), xi = ld<T, kIn<T>>(sp, P, p, SLOT_C2(4) + 1);
         const T yr = ld<T, kIn<T>>(sp, P, p, SLOT_R0(14)), yi = ld<T, kIn<T>>(sp, P, p, SLOT_R0(15));
-        Prm[1][0] = half * (xr + yr);
-        Prm[1][1] = half * (xi - yi);
-        Prm[2][0] = half * (xi + yi);
-        Prm[2][1] = half * (yr - xr);
+        Prm[1][0] = half_of(xr + yr);
+        Prm[1][1] = half_of(xi - yi);
+        Prm[2][0] = half_of(xi + yi);
+        Prm[2][1] = half_of(yr - xr);
       }
       {
         // X = (m; mm) = P^th + i P^ph, Z = (mbar; mm) = P^th - i P^ph
         const T xr = ld<T, kIn<T>>(sp, P, p, SLOT_C3), xi = ld<T, kIn<T>>(sp, P, p, SLOT_C3 + 1);
         const T zr = ld<T, kIn<T>>(sp, P, p, SLOT_C1(10)), zi = ld<T, kIn<T>>(sp, P, p, SLOT_C1(10) + 1);
-        Pmm[1][0] = half * (xr + zr);
-        Pmm[1][1] = half * (xi + zi);
-        Pmm[2][0] = half * (xi - zi);
-        Pmm[2][1] = half * (zr - xr);
+        Pmm[1][0] = half_of(xr + zr);
+        Pmm[1][1] = half_of(xi + zi);
+        Pmm[2][0] = half_of(xi - zi);
+        Pmm[2][1] = half_of(zr - xr);
       }
       // slots 6 A + q: the pair part Trot_A of triad leg A (q: rr, r1, r2,
       // 11, 12, 22), then in its place X_A, the pair back in Cartesian
@@ -439,9 +437,9 @@ __device__ __forceinline__ void reconstruct_group(int grp, Scratch<T> sc, const 
         sc(6 * A + 0) = Pr[A];
         sc(6 * A + 1) = Prm[A][0];
         sc(6 * A + 2) = Prm[A][1];
-        sc(6 * A + 3) = half * (Pmb[A] + Pmm[A][0]);
-        sc(6 * A + 4) = half * Pmm[A][1];
-        sc(6 * A + 5) = half * (Pmb[A] - Pmm[A][0]);
+        sc(6 * A + 3) = half_of(Pmb[A] + Pmm[A][0]);
+        sc(6 * A + 4) = half_of(Pmm[A][1]);
+        sc(6 * A + 5) = half_of(Pmb[A] - Pmm[A][0]);
       }
 #pragma unroll 1
       for (int A = 0; A < 3; ++A) {
@@ -540,7 +538,7 @@ __device__ __forceinline__ void reconstruct_update(Scratch<T> sc, const double* 
       bad |= !finite_s(k);
       // stage state: FP64 sum on the FP64 path, double-float on the mixed path
       const T base = kPair ? SI_::ld(uf, o) : S<T>::c(u[o]);
-      SI_::st(kacc, o, stage == 0 ? k : SI_::ld(kacc, o) + (k + k));
+      SI_::st(kacc, o, stage == 0 ? k : SI_::ld(kacc, o) + twice(k));
       SI_::st(U, o, base + cU * k);
     } else {
       bad |= !finite_s(k);
@@ -647,7 +645,6 @@ __device__ __forceinline__ Share share_of(const Geo& geo) {
 template <class T, class Emit>
 __device__ __forceinline__ void reconstruct_rank3(int w, PointScratch<T> sc, const double* __restrict__ sp, long long P,
                                                   long long p, const Triad<T>& t, Emit&& emit) {
-  const T half = S<T>::c(0.5);
   auto in = [&](int slot) { return ld<T, kIn<T>>(sp, P, p, slot); };
   T pr, pmb, prm0, prm1, pmm0, pmm1;
   if (w == 0) {
@@ -665,15 +662,15 @@ __device__ __forceinline__ void reconstruct_rank3(int w, PointScratch<T> sc, con
     // X' = (m; mm) = P^th + i P^ph, Z = (mbar; mm) = P^th - i P^ph
     const T mr = in(SLOT_C3), mi = in(SLOT_C3 + 1), zr = in(SLOT_C1(10)), zi = in(SLOT_C1(10) + 1);
     if (w == 1) {
-      prm0 = half * (xr + yr);
-      prm1 = half * (xi - yi);
-      pmm0 = half * (mr + zr);
-      pmm1 = half * (mi + zi);
+      prm0 = half_of(xr + yr);
+      prm1 = half_of(xi - yi);
+      pmm0 = half_of(mr + zr);
+      pmm1 = half_of(mi + zi);
     } else {
-      prm0 = half * (xi + yi);
-      prm1 = half * (yr - xr);
-      pmm0 = half * (mi - zi);
-      pmm1 = half * (zr - mr);
+      prm0 = half_of(xi + yi);
+      prm1 = half_of(yr - xr);
+      pmm0 = half_of(mi - zi);
+      pmm1 = half_of(zr - mr);
     }
   }
   {
@@ -681,9 +678,9 @@ __device__ __forceinline__ void reconstruct_rank3(int w, PointScratch<T> sc, con
     Trot[0][0] = pr;
     Trot[0][1] = prm0;
     Trot[0][2] = prm1;
-    Trot[1][1] = half * (pmb + pmm0);
-    Trot[1][2] = half * pmm1;
-    Trot[2][2] = half * (pmb - pmm0);
+    Trot[1][1] = half_of(pmb + pmm0);
+    Trot[1][2] = half_of(pmm1);
+    Trot[2][2] = half_of(pmb - pmm0);
     unrot_sym(t, Trot, X);
 #pragma unroll
     for (int b = 0; b < 3; ++b)
@@ -749,7 +746,7 @@ struct StageUpdate {
       if (kPair && uf) SI_::st(uf, o, k);
     } else if (KIND == 1) {
       bad |= !finite_s(k);
-      const T acc = stage == 0 ? k : x.acc + (k + k), un = x.base + cU * k;
+      const T acc = stage == 0 ? k : x.acc + twice(k), un = x.base + cU * k;
       if (!live) return;
       SI_::st(kacc, o, acc);
       SI_::st(U, o, un);

@@ -134,14 +134,13 @@ __device__ __forceinline__ void christoffel(const Metric<T>& M, const T Pi[10], 
 #pragma unroll
     for (int i = 0; i < 3; ++i) dg4[i + 1][s] = Ph[i][s];
   }
-  const T half = S<T>::c(0.5);
 #pragma unroll
   for (int c = 0; c < 4; ++c)
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int b = a; b < 4; ++b)
-        Gam[c][SI(a, b)] = half * (dg4[a][SI(b, c)] + dg4[b][SI(a, c)] - dg4[c][SI(a, b)]);
+        Gam[c][SI(a, b)] = half_of(dg4[a][SI(b, c)] + dg4[b][SI(a, c)] - dg4[c][SI(a, b)]);
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     T acc = S<T>::c(0.0);

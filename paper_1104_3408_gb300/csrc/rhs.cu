@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
   const long long P = geo.P;
   const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (p >= P) return;
-  const T zero = S<T>::c(0.0), half = S<T>::c(0.5);
+  const T zero = S<T>::c(0.0);
 
   Metric<T> M;
   {
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = a; b < 4; ++b)
-          V(c * 10 + SI(a, b)) = half * (dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
+          V(c * 10 + SI(a, b)) = half_of(dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
   }
   // Gamma_c = g^ab Gamma_cab (symmetric pairs counted twice off the diagonal);
   // gauge constraint C_c = H_c + Gamma_c, H^c, n^c C_c
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = a; b < 4; ++b) {
-          const T w = (a == b) ? M.gi4[SI(a, b)] : M.gi4[SI(a, b)] + M.gi4[SI(a, b)];
+          const T w = (a == b) ? M.gi4[SI(a, b)] : twice(M.gi4[SI(a, b)]);
           acc.fma_(w, V(c * 10 + SI(a, b)));
         }
       const T hc = c == 0 ? Hd[0] : (c == 1 ? Hd[1] : (c == 2 ? Hd[2] : Hd[3]));
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
       const T dHba = b == 0 ? (dtH ? ldA<T, kInt<T>>(dH, P, p, 12 + a) : zero)
                             : ldA<T, kInt<T>>(dH, P, p, (b - 1) * 4 + a);
       Acc<T> acc;
-      acc.fma_(half, dHab + dHba);
+      acc.add(half_of(dHab + dHba));
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc.fma_(-V(c * 10 + s), Hup[c]);
       const T DH = acc.get();
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
             Acc<T> acc;
 #pragma unroll
             for (int f = 0; f < 4; ++f) acc.fma_(M.gi4[SI(e, f)], Gcf[c][f]);
-            Gce[SI(c, e)] = (c == e) ? acc.get() : acc.get() + acc.get();
+            Gce[SI(c, e)] = (c == e) ? acc.get() : twice(acc.get());
           }
       }
 #pragma unroll 1
@@ -228,7 +228,6 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
   const long long P = geo.P;
   const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (p >= P) return;
-  const T half = S<T>::c(0.5);
   // 3+1 quantities (eqs. normal, abgfromgab) as k_rhs_gamma derived them
   const T alpha = ldA<T, kInt<T>>(src, P, p, 40);
   T bu[3], gi[3][3];
@@ -344,7 +343,7 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
       cPh[y] = bu[y] - alpha * acc.get();
     }
   }
-  const T hal = half * alpha;
+  const T hal = half_of(alpha);
   const T cPi = -(hal * nnPi);
 #pragma unroll 1
   for (int s = 0; s < 10; ++s) {
@@ -430,7 +429,7 @@ __global__ void __launch_bounds__(kRhsBlock)
   const long long q = blockIdx.x * 32ll + lane;
   const bool live = q < P;
   const long long p = live ? q : P - 1;  // the last block's spare threads follow its last point
-  const T zero = S<T>::c(0.0), half = S<T>::c(0.5);
+  const T zero = S<T>::c(0.0);
 
   if (w == 0) {
     T g[10];
@@ -500,9 +499,9 @@ __global__ void __launch_bounds__(kRhsBlock)
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int b = a; b < 4; ++b) {
-        const T G = half * (dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
+        const T G = half_of(dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
         V(kGGam + c * 10 + SI(a, b)) = G;
-        const T wt = (a == b) ? gi4[SI(a, b)] : gi4[SI(a, b)] + gi4[SI(a, b)];
+        const T wt = (a == b) ? gi4[SI(a, b)] : twice(gi4[SI(a, b)]);
         acc.fma_(wt, G);
       }
     acc.add(c == 0 ? Hd[0] : (c == 1 ? Hd[1] : (c == 2 ? Hd[2] : Hd[3])));
@@ -544,7 +543,7 @@ __global__ void __launch_bounds__(kRhsBlock)
         Acc<T> acc;
 #pragma unroll
         for (int f = 0; f < 4; ++f) acc.fma_(gi4[SI(e, f)], Gcf[c][f]);
-        Gce[SI(c, e)] = (c == e) ? acc.get() : acc.get() + acc.get();
+        Gce[SI(c, e)] = (c == e) ? acc.get() : twice(acc.get());
       }
   }
   const T twoal = alpha + alpha, m2al = -twoal;
@@ -563,7 +562,7 @@ __global__ void __launch_bounds__(kRhsBlock)
                           : ldA<T, kInt<T>>(dH, P, p, (b - 1) * 4 + a);
     const T gab = ldA<T, FU>(u, P, p, s);
     Acc<T> acc;
-    acc.fma_(half, dHab + dHba);
+    acc.add(half_of(dHab + dHba));
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc.fma_(-V(kGGam + c * 10 + s), Hup[c]);
     const T DH = acc.get();
@@ -601,7 +600,6 @@ __global__ void __launch_bounds__(kRhsBlock)
   const long long q = blockIdx.x * 32ll + lane;
   const bool live = q < P;
   const long long p = live ? q : P - 1;
-  const T half = S<T>::c(0.5);
   {
     T v[13];
 #pragma unroll
@@ -633,7 +631,7 @@ __global__ void __launch_bounds__(kRhsBlock)
   nu[0] = ialpha;
 #pragma unroll
   for (int i = 0; i < 3; ++i) nu[i + 1] = -(bu[i] * ialpha);
-  const T hal = half * alpha;
+  const T hal = half_of(alpha);
   {
     T gi4[10];
     gi4[0] = -ia2;
@@ -811,7 +809,6 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   fetch(s0);
-  const T half = S<T>::c(0.5);
   const Jac<T> J = jacobian<T>(geo, k, i, jj);
   const T alpha = ldA<T, kInt<T>>(src, P, p, 40);
   T bu[3], gi[3][3];
@@ -909,8 +906,8 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
 #pragma unroll
       for (int x = 0; x < 3; ++x) sd.fma_(su[x], rPh[x]);
       const T wplus = rPi + sd.get();
-      const T w2 = half * (wplus - rg);
-      rPi = half * (rg + wplus);
+      const T w2 = half_of(wplus - rg);
+      rPi = half_of(rg + wplus);
 #pragma unroll
       for (int x = 0; x < 3; ++x) rPh[x] = sl[x] * w2;
     }
