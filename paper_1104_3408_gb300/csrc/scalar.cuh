@@ -194,7 +194,9 @@ __device__ __forceinline__ ff twice(ff x) { return ff{fa(x.hi, x.hi), fa(x.lo, x
 // SIAM J. Sci. Comput. 26 (2005)): every product is split exactly by TwoProd
 // (with the cross terms of the low parts folded in), the running sum by
 // TwoSum, and all error terms collect in one FP32 word that is added back at
-// the end.
+// the end.  The first term needs no TwoSum: s and c are its two words, 4
+// instructions for a product (each later one takes 12) and none for a term; the
+// loops over the terms are unrolled, so that `first` costs nothing.
 template <class T> struct Acc;
 template <> struct Acc<double> {
   double s = 0.0;
@@ -204,24 +206,28 @@ template <> struct Acc<double> {
 };
 template <> struct Acc<ff> {
   float s = 0.0f, c = 0.0f;
-  __device__ __forceinline__ void fma_(ff a, ff b) {
-    const float p = fm(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
+  bool first = true;
+  // one more term p + e, e of the size of an error of p
+  __device__ __forceinline__ void term(float p, float e) {
+    if (first) {
+      s = p;
+      c = e;
+      first = false;
+      return;
+    }
     const float t = fa(s, p);
     const float bb = fs(t, s);
     const float err = fa(fs(s, fs(t, bb)), fs(p, bb));
     s = t;
     c = fa(c, fa(err, e));
   }
-  __device__ __forceinline__ void add(ff a) {
-    const float t = fa(s, a.hi);
-    const float bb = fs(t, s);
-    const float err = fa(fs(s, fs(t, bb)), fs(a.hi, bb));
-    s = t;
-    c = fa(c, fa(err, a.lo));
+  __device__ __forceinline__ void fma_(ff a, ff b) {
+    const float p = fm(a.hi, b.hi);
+    float e = fmaf(a.hi, b.hi, -p);
+    e = fmaf(a.hi, b.lo, e);
+    term(p, fmaf(a.lo, b.hi, e));
   }
+  __device__ __forceinline__ void add(ff a) { term(a.hi, a.lo); }
   __device__ __forceinline__ ff get() const { return two_sum(s, c); }
 };
 
