@@ -23,6 +23,14 @@ __host__ __device__ __forceinline__ constexpr int SI(int a, int b) {
   return lo == 0 ? hi : (lo == 1 ? 3 + hi : (lo == 2 ? 5 + hi : 9));
 }
 
+// SI(a, .) of a row a known only at run time: the row's four indices in 16 bits (the
+// selects of SI take three times the instructions)
+struct SymRow {
+  unsigned r;
+  __device__ __forceinline__ explicit SymRow(int a) : r((unsigned)(0x9863875265413210ull >> (16 * a))) {}
+  __device__ __forceinline__ int operator()(int c) const { return (int)((r >> (4 * c)) & 15u); }
+};
+
 template <class T>
 struct Jac {
   // d/dx^k = J[k][0] d_r + J[k][1] d_theta + J[k][2] d_phi

@@ -263,25 +263,28 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
   // Q = Q1 - Q2 into slots 40..49; Q2_ab = Pi_ac g^cd Pi_db
 #pragma unroll 1
   for (int b = 0; b < 4; ++b) {
+    const SymRow rb(b);
     T Piu[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       Acc<T> acc;
 #pragma unroll
-      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(SI(b, d)));
+      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(rb(d)));
       Piu[c] = acc.get();
     }
 #pragma unroll 1
     for (int a = 0; a <= b; ++a) {
+      const SymRow ra(a);
       Acc<T> acc;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc.fma_(-V(SI(a, c)), Piu[c]);
-      V(40 + SI(a, b)) = acc.get();
+      for (int c = 0; c < 4; ++c) acc.fma_(-V(ra(c)), Piu[c]);
+      V(40 + rb(a)) = acc.get();
     }
   }
   // Q1_ab = gamma^ij g^cd Phi_iac Phi_jbd
 #pragma unroll 1
   for (int b = 0; b < 4; ++b) {
+    const SymRow rb(b);
     T W[3][4];
     {
       T Y[3][4];
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
         for (int c = 0; c < 4; ++c) {
           Acc<T> acc;
 #pragma unroll
-          for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(10 + 10 * x + SI(b, d)));
+          for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(10 + 10 * x + rb(d)));
           Y[x][c] = acc.get();
         }
 #pragma unroll
@@ -306,13 +309,14 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
     }
 #pragma unroll 1
     for (int a = 0; a <= b; ++a) {
+      const SymRow ra(a);
       Acc<T> acc;
-      acc.add(V(40 + SI(a, b)));
+      acc.add(V(40 + rb(a)));
 #pragma unroll
       for (int x = 0; x < 3; ++x)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc.fma_(V(10 + 10 * x + SI(a, c)), W[x][c]);
-      V(40 + SI(a, b)) = acc.get();
+        for (int c = 0; c < 4; ++c) acc.fma_(V(10 + 10 * x + ra(c)), W[x][c]);
+      V(40 + rb(a)) = acc.get();
     }
   }
   // remaining algebraic terms of eq. Pidot
