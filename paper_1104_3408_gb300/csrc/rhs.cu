@@ -178,6 +178,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
     const T m2al = -(M.alpha + M.alpha);
 #pragma unroll 1
     for (int b = 0; b < 4; ++b) {
+      const SymRow rb(b);
       T Gce[10];  // Gamma_b^{ce}, symmetric, off-diagonal weight 2
       {
         T Gcf[4][4];  // Gamma_b^c_f = g^cd Gamma_bdf
@@ -208,9 +209,10 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
 #pragma unroll
           for (int e = c; e < 4; ++e) qa.fma_(V(a * 10 + SI(c, e)), Gce[SI(c, e)]);
         Acc<T> acc;
-        acc.add(V(40 + SI(a, b)));
+        const int s = 40 + rb(a);
+        acc.add(V(s));
         acc.fma_(m2al, qa.get());
-        V(40 + SI(a, b)) = acc.get();
+        V(s) = acc.get();
       }
     }
   }
@@ -528,6 +530,7 @@ __global__ void __launch_bounds__(kRhsBlock)
   }
   // the sources with larger index b = w
   const int b = w;
+  const SymRow rb(b);
   T Gce[10];  // Gamma_b^{ce}, symmetric, off-diagonal weight 2
   {
     T Gcf[4][4];  // Gamma_b^c_f = g^cd Gamma_bdf
@@ -555,7 +558,7 @@ __global__ void __launch_bounds__(kRhsBlock)
   const T anC = alpha * nC;
 #pragma unroll 1
   for (int a = 0; a <= b; ++a) {
-    const int s = SI(a, b);
+    const int s = rb(a);
     // S_Pi = -2 alpha nabla_(a H_b) + alpha (n_b C_a + n_a C_b - g_ab n^c C_c);
     // d_a H_b: rows (x, b) = 4 x + b of dH for a = x + 1; d_t H_b is row 12 + b
     // when the gauge source is evolved with its time derivative (58 fields),
@@ -647,13 +650,14 @@ __global__ void __launch_bounds__(kRhsBlock)
       for (int j = i; j < 3; ++j) gi4[SI(i + 1, j + 1)] = gi[i][j] - bu[i] * bu[j] * ia2;
     const T twoal = alpha + alpha;
     const int b = w;
+    const SymRow rb(b);
     // Q2_ab = Pi_ac g^cd Pi_db, Q1_ab = gamma^ij g^cd Phi_iac Phi_jbd
     T Piu[4], W[3][4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       Acc<T> acc;
 #pragma unroll
-      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kQPi + SI(b, d)));
+      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kQPi + rb(d)));
       Piu[c] = acc.get();
     }
     {
@@ -664,7 +668,7 @@ __global__ void __launch_bounds__(kRhsBlock)
         for (int c = 0; c < 4; ++c) {
           Acc<T> acc;
 #pragma unroll
-          for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kQPh + 10 * x + SI(b, d)));
+          for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(kQPh + 10 * x + rb(d)));
           Y[x][c] = acc.get();
         }
 #pragma unroll
@@ -708,17 +712,18 @@ __global__ void __launch_bounds__(kRhsBlock)
     const T cPi = -(hal * nnPi);
 #pragma unroll 1
     for (int a = 0; a <= b; ++a) {
-      const int s = SI(a, b);
+      const SymRow ra(a);
+      const int s = rb(a);
       const T part = ldA<T, kInt<T>>(src, P, p, s);
       Acc<T> q2;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) q2.fma_(-V(kQPi + SI(a, c)), Piu[c]);
+      for (int c = 0; c < 4; ++c) q2.fma_(-V(kQPi + ra(c)), Piu[c]);
       Acc<T> qq;
       qq.add(q2.get());
 #pragma unroll
       for (int x = 0; x < 3; ++x)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) qq.fma_(V(kQPh + 10 * x + SI(a, c)), W[x][c]);
+        for (int c = 0; c < 4; ++c) qq.fma_(V(kQPh + 10 * x + ra(c)), W[x][c]);
       Acc<T> acc;
       acc.add(part);
       acc.fma_(twoal, qq.get());
