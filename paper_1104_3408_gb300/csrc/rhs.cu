@@ -51,6 +51,32 @@ struct Slots {
   __device__ __forceinline__ T& operator()(int v) const { return s[v * NB + (int)threadIdx.x]; }
 };
 
+// Gamma_cab = (d_a g_bc + d_b g_ac - d_c g_ab) / 2; dg4(c, s) = d_c g of pair s.  The
+// terms that cancel or are equal are not summed: 500 instructions for the 40
+// symbols of a point, not 960.
+template <class T, class DG>
+__device__ __forceinline__ T gamma_cab(int c, int a, int b, DG&& dg4) {
+  if (c == a) return half_of(dg4(b, SI(a, a)));
+  if (c == b) return half_of(dg4(a, SI(b, b)));
+  const T two = a == b ? twice(dg4(a, SI(a, c))) : dg4(a, SI(b, c)) + dg4(b, SI(a, c));
+  return half_of(two - dg4(c, SI(a, b)));
+}
+
+// n^d A_cd of a symmetric A(pair) for all c, and n^c n^d A_cd
+template <class T, class A>
+__device__ __forceinline__ T normal_row(const T (&nu)[4], T (&row)[4], A&& pair) {
+  Acc<T> nn;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    Acc<T> acc;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) acc.fma_(nu[d], pair(SI(c, d)));
+    row[c] = acc.get();
+    nn.fma_(nu[c], row[c]);
+  }
+  return nn.get();
+}
+
 constexpr int kRhsBlock = 128;
 constexpr int kGamSlots = 54;   // Gamma_cab (c*10 + s) | S_Pi 40..49 | C_a 50..53
 constexpr int kQuadSlots = 50;  // Pi 0..9 | Phi_iab 10 + 10 i + s | Q 40..49
@@ -110,7 +136,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = a; b < 4; ++b)
-          V(c * 10 + SI(a, b)) = half_of(dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
+          V(c * 10 + SI(a, b)) = gamma_cab<T>(c, a, b, dg4);
   }
   // Gamma_c = g^ab Gamma_cab (symmetric pairs counted twice off the diagonal);
   // gauge constraint C_c = H_c + Gamma_c, H^c, n^c C_c
@@ -322,30 +348,15 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
     }
   }
   // remaining algebraic terms of eq. Pidot
-  T nnPi;
+  T nnPi, cPh[3];  // n^c n^d Pi_cd; beta^j - alpha n^c Pi_ci gamma^ij
   {
-    Acc<T> acc;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int d = 0; d < 4; ++d) acc.fma_(nu[c] * nu[d], V(SI(c, d)));
-    nnPi = acc.get();
-  }
-  T cPh[3];  // beta^j - alpha n^c Pi_ci gamma^ij
-  {
-    T nPi[3];
-#pragma unroll
-    for (int x = 0; x < 3; ++x) {
-      Acc<T> acc;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc.fma_(nu[c], V(SI(c, x + 1)));
-      nPi[x] = acc.get();
-    }
+    T nPi[4];
+    nnPi = normal_row(nu, nPi, [&](int s) -> T { return V(s); });
 #pragma unroll
     for (int y = 0; y < 3; ++y) {
       Acc<T> acc;
 #pragma unroll
-      for (int x = 0; x < 3; ++x) acc.fma_(nPi[x], gi[x][y]);
+      for (int x = 0; x < 3; ++x) acc.fma_(nPi[x + 1], gi[x][y]);
       cPh[y] = bu[y] - alpha * acc.get();
     }
   }
@@ -364,31 +375,17 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
   // algebraic terms of eq. Phidot
 #pragma unroll 1
   for (int x = 0; x < 3; ++x) {
-    T nnPhi;
+    T nnPhi, Mk[3];  // n^c n^d Phi_xcd; alpha gamma^jk n^c Phi_x,j,c less alpha delta^k_x
     {
-      Acc<T> acc;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int d = 0; d < 4; ++d) acc.fma_(nu[c] * nu[d], V(10 + 10 * x + SI(c, d)));
-      nnPhi = acc.get();
-    }
-    T Mk[3];  // alpha gamma^jk n^c Phi_x,j,c
-    {
-      T nP[3];
-#pragma unroll
-      for (int y = 0; y < 3; ++y) {
-        Acc<T> acc;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc.fma_(nu[c], V(10 + 10 * x + SI(y + 1, c)));
-        nP[y] = acc.get();
-      }
+      T nP[4];
+      nnPhi = normal_row(nu, nP, [&](int s) -> T { return V(10 + 10 * x + s); });
 #pragma unroll
       for (int z = 0; z < 3; ++z) {
         Acc<T> acc;
 #pragma unroll
-        for (int y = 0; y < 3; ++y) acc.fma_(nP[y], gi[y][z]);
+        for (int y = 0; y < 3; ++y) acc.fma_(nP[y + 1], gi[y][z]);
         Mk[z] = alpha * acc.get();
+        if (z == x) Mk[z] = Mk[z] - alpha;
       }
     }
     const T hnn = hal * nnPhi;
@@ -398,7 +395,6 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
       acc.fma_(hnn, V(s));
 #pragma unroll
       for (int z = 0; z < 3; ++z) acc.fma_(Mk[z], V(10 + 10 * z + s));
-      acc.fma_(-alpha, V(10 + 10 * x + s));
       stA<T, kInt<T>>(src, P, p, 10 + 10 * x + s, acc.get());
     }
   }
@@ -505,7 +501,7 @@ __global__ void __launch_bounds__(kRhsBlock)
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int b = a; b < 4; ++b) {
-        const T G = half_of(dg4(a, SI(b, c)) + dg4(b, SI(a, c)) - dg4(c, SI(a, b)));
+        const T G = gamma_cab<T>(c, a, b, dg4);
         V(kGGam + c * 10 + SI(a, b)) = G;
         const T wt = (a == b) ? gi4[SI(a, b)] : twice(gi4[SI(a, b)]);
         acc.fma_(wt, G);
@@ -682,30 +678,15 @@ __global__ void __launch_bounds__(kRhsBlock)
         }
     }
     // remaining algebraic terms of eq. Pidot
-    T nnPi;
+    T nnPi, cPh[3];  // n^c n^d Pi_cd; beta^j - alpha n^c Pi_ci gamma^ij
     {
-      Acc<T> acc;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int d = 0; d < 4; ++d) acc.fma_(nu[c] * nu[d], V(kQPi + SI(c, d)));
-      nnPi = acc.get();
-    }
-    T cPh[3];  // beta^j - alpha n^c Pi_ci gamma^ij
-    {
-      T nPi[3];
-#pragma unroll
-      for (int x = 0; x < 3; ++x) {
-        Acc<T> acc;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc.fma_(nu[c], V(kQPi + SI(c, x + 1)));
-        nPi[x] = acc.get();
-      }
+      T nPi[4];
+      nnPi = normal_row(nu, nPi, [&](int s) -> T { return V(kQPi + s); });
 #pragma unroll
       for (int y = 0; y < 3; ++y) {
         Acc<T> acc;
 #pragma unroll
-        for (int x = 0; x < 3; ++x) acc.fma_(nPi[x], gi[x][y]);
+        for (int x = 0; x < 3; ++x) acc.fma_(nPi[x + 1], gi[x][y]);
         cPh[y] = bu[y] - alpha * acc.get();
       }
     }
@@ -736,31 +717,17 @@ __global__ void __launch_bounds__(kRhsBlock)
   if (w == 3) return;
   // algebraic terms of eq. Phidot
   const int x = w;
-  T nnPhi;
+  T nnPhi, Mk[3];  // n^c n^d Phi_xcd; alpha gamma^jk n^c Phi_x,j,c less alpha delta^k_x
   {
-    Acc<T> acc;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int d = 0; d < 4; ++d) acc.fma_(nu[c] * nu[d], V(kQPh + 10 * x + SI(c, d)));
-    nnPhi = acc.get();
-  }
-  T Mk[3];  // alpha gamma^jk n^c Phi_x,j,c
-  {
-    T nP[3];
-#pragma unroll
-    for (int y = 0; y < 3; ++y) {
-      Acc<T> acc;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc.fma_(nu[c], V(kQPh + 10 * x + SI(y + 1, c)));
-      nP[y] = acc.get();
-    }
+    T nP[4];
+    nnPhi = normal_row(nu, nP, [&](int s) -> T { return V(kQPh + 10 * x + s); });
 #pragma unroll
     for (int z = 0; z < 3; ++z) {
       Acc<T> acc;
 #pragma unroll
-      for (int y = 0; y < 3; ++y) acc.fma_(nP[y], gi[y][z]);
+      for (int y = 0; y < 3; ++y) acc.fma_(nP[y + 1], gi[y][z]);
       Mk[z] = alpha * acc.get();
+      if (z == x) Mk[z] = Mk[z] - alpha;
     }
   }
   const T hnn = hal * nnPhi;
@@ -770,7 +737,6 @@ __global__ void __launch_bounds__(kRhsBlock)
     acc.fma_(hnn, V(kQPi + s));
 #pragma unroll
     for (int z = 0; z < 3; ++z) acc.fma_(Mk[z], V(kQPh + 10 * z + s));
-    acc.fma_(-alpha, V(kQPh + 10 * x + s));
     if (live) stA<T, kInt<T>>(src, P, p, 10 + 10 * x + s, acc.get());
   }
 }
@@ -905,7 +871,7 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
         a.fma_(b[m], DPh[x][m]);
-        a.fma_(aJ[x][m], Dd[m]);
+        if (x < 2 || m < 2) a.fma_(aJ[x][m], Dd[m]);  // z does not depend on phi
       }
       rPh[x] = a.get();
     }
