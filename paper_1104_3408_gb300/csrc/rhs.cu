@@ -79,7 +79,7 @@ __device__ __forceinline__ T normal_row(const T (&nu)[4], T (&row)[4], A&& pair)
 
 constexpr int kRhsBlock = 128;
 constexpr int kGamSlots = 54;   // Gamma_cab (c*10 + s) | S_Pi 40..49 | C_a 50..53
-constexpr int kQuadSlots = 50;  // Pi 0..9 | Phi_iab 10 + 10 i + s | Q 40..49
+constexpr int kQuadSlots = 40;  // Pi 0..9 | Phi_iab 10 + 10 i + s
 
 // Four blocks per SM: 128 registers, 54 KB of slots (g_ab is read again from
 // u where the gauge terms need it instead of holding ten more slots).
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
 // The Phi-Phi and Pi-Pi terms of eq. Pidot and the remaining algebraic terms
 // of eqs. Pidot and Phidot; alpha, beta^i, gamma^ij come from k_rhs_gamma.
 template <class T, bool FU>
-__global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict__ u, double* __restrict__ src,
+__global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_quad(const double* __restrict__ u, double* __restrict__ src,
                                                         Geo geo) {
   __shared__ T sm[kQuadSlots * kRhsBlock];
   const Slots<T, kRhsBlock> V{sm};
@@ -288,89 +288,71 @@ __global__ void __launch_bounds__(kRhsBlock) k_rhs_quad(const double* __restrict
     for (int x = 0; x < 3; ++x) V(10 + 10 * x + s) = ldA<T, FU>(u, P, p, 20 + 10 * x + s);
   }
   const T twoal = alpha + alpha;
-  // Q = Q1 - Q2 into slots 40..49; Q2_ab = Pi_ac g^cd Pi_db
-#pragma unroll 1
-  for (int b = 0; b < 4; ++b) {
-    const SymRow rb(b);
-    T Piu[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      Acc<T> acc;
-#pragma unroll
-      for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(rb(d)));
-      Piu[c] = acc.get();
-    }
-#pragma unroll 1
-    for (int a = 0; a <= b; ++a) {
-      const SymRow ra(a);
-      Acc<T> acc;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc.fma_(-V(ra(c)), Piu[c]);
-      V(40 + rb(a)) = acc.get();
-    }
-  }
-  // Q1_ab = gamma^ij g^cd Phi_iac Phi_jbd
-#pragma unroll 1
-  for (int b = 0; b < 4; ++b) {
-    const SymRow rb(b);
-    T W[3][4];
-    {
-      T Y[3][4];
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          Acc<T> acc;
-#pragma unroll
-          for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(10 + 10 * x + rb(d)));
-          Y[x][c] = acc.get();
-        }
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          Acc<T> acc;
-#pragma unroll
-          for (int y = 0; y < 3; ++y) acc.fma_(gi[x][y], Y[y][c]);
-          W[x][c] = acc.get();
-        }
-    }
-#pragma unroll 1
-    for (int a = 0; a <= b; ++a) {
-      const SymRow ra(a);
-      Acc<T> acc;
-      acc.add(V(40 + rb(a)));
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc.fma_(V(10 + 10 * x + ra(c)), W[x][c]);
-      V(40 + rb(a)) = acc.get();
-    }
-  }
-  // remaining algebraic terms of eq. Pidot
-  T nnPi, cPh[3];  // n^c n^d Pi_cd; beta^j - alpha n^c Pi_ci gamma^ij
-  {
-    T nPi[4];
-    nnPi = normal_row(nu, nPi, [&](int s) -> T { return V(s); });
-#pragma unroll
-    for (int y = 0; y < 3; ++y) {
-      Acc<T> acc;
-#pragma unroll
-      for (int x = 0; x < 3; ++x) acc.fma_(nPi[x + 1], gi[x][y]);
-      cPh[y] = bu[y] - alpha * acc.get();
-    }
-  }
   const T hal = half_of(alpha);
-  const T cPi = -(hal * nnPi);
-#pragma unroll 1
-  for (int s = 0; s < 10; ++s) {
-    Acc<T> acc;
-    acc.add(ldA<T, kInt<T>>(src, P, p, s));
-    acc.fma_(twoal, V(40 + s));
-    acc.fma_(cPi, V(s));
+  {
+    T nnPi, cPh[3];  // n^c n^d Pi_cd; beta^j - alpha n^c Pi_ci gamma^ij
+    {
+      T nPi[4];
+      nnPi = normal_row(nu, nPi, [&](int s) -> T { return V(s); });
 #pragma unroll
-    for (int x = 0; x < 3; ++x) acc.fma_(cPh[x], V(10 + 10 * x + s));
-    stA<T, kInt<T>>(src, P, p, s, acc.get());
+      for (int y = 0; y < 3; ++y) {
+        Acc<T> acc;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) acc.fma_(nPi[x + 1], gi[x][y]);
+        cPh[y] = bu[y] - alpha * acc.get();
+      }
+    }
+    const T cPi = -(hal * nnPi);
+    // the sources with larger index b: Q2_ab = Pi_ac g^cd Pi_db, Q1_ab = gamma^ij
+    // g^cd Phi_iac Phi_jbd and the remaining algebraic terms of eq. Pidot
+#pragma unroll 1
+    for (int b = 0; b < 4; ++b) {
+      const SymRow rb(b);
+      T Piu[4], W[3][4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        Acc<T> acc;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) acc.fma_(gi4[SI(c, d)], V(rb(d)));
+        Piu[c] = acc.get();
+        T Y[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          Acc<T> ay;
+#pragma unroll
+          for (int d = 0; d < 4; ++d) ay.fma_(gi4[SI(c, d)], V(10 + 10 * x + rb(d)));
+          Y[x] = ay.get();
+        }
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          Acc<T> aw;
+#pragma unroll
+          for (int y = 0; y < 3; ++y) aw.fma_(gi[x][y], Y[y]);
+          W[x][c] = aw.get();
+        }
+      }
+#pragma unroll 1
+      for (int a = 0; a <= b; ++a) {
+        const SymRow ra(a);
+        const int s = rb(a);
+        Acc<T> q2;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q2.fma_(-V(ra(c)), Piu[c]);
+        Acc<T> q;
+        q.add(q2.get());
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) q.fma_(V(10 + 10 * x + ra(c)), W[x][c]);
+        Acc<T> acc;
+        acc.add(ldA<T, kInt<T>>(src, P, p, s));
+        acc.fma_(twoal, q.get());
+        acc.fma_(cPi, V(s));
+#pragma unroll
+        for (int x = 0; x < 3; ++x) acc.fma_(cPh[x], V(10 + 10 * x + s));
+        stA<T, kInt<T>>(src, P, p, s, acc.get());
+      }
+    }
   }
   // algebraic terms of eq. Phidot
 #pragma unroll 1
