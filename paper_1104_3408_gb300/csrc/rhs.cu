@@ -78,7 +78,7 @@ __device__ __forceinline__ T normal_row(const T (&nu)[4], T (&row)[4], A&& pair)
 }
 
 constexpr int kRhsBlock = 128;
-constexpr int kGamSlots = 54;   // Gamma_cab (c*10 + s) | S_Pi 40..49 | C_a 50..53
+constexpr int kGamSlots = 44;   // Gamma_cab (c*10 + s) | C_a 40..43
 constexpr int kQuadSlots = 40;  // Pi 0..9 | Phi_iab 10 + 10 i + s
 
 // Four blocks per SM: 128 registers, 54 KB of slots (g_ab is read again from
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
         }
       const T hc = c == 0 ? Hd[0] : (c == 1 ? Hd[1] : (c == 2 ? Hd[2] : Hd[3]));
       acc.add(hc);
-      V(50 + c) = acc.get();
+      V(40 + c) = acc.get();
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -166,26 +166,54 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
 #pragma unroll
       for (int d = 0; d < 4; ++d) acc.fma_(M.gi4[SI(c, d)], Hd[d]);
       Hup[c] = acc.get();
-      an.fma_(M.nu[c], V(50 + c));
+      an.fma_(M.nu[c], V(40 + c));
     }
     nC = an.get();
   }
-  // S_Pi = -2 alpha nabla_(a H_b) + alpha (n_b C_a + n_a C_b - g_ab n^c C_c)
-  {
-    const T twoal = M.alpha + M.alpha;
-    const T aa = M.alpha * (-M.alpha);  // alpha n_0, n_a = (-alpha, 0, 0, 0)
-    const T anC = M.alpha * nC;
+  // the sources with larger index b
+  const T twoal = M.alpha + M.alpha, m2al = -twoal;
+  const T aa = M.alpha * (-M.alpha);  // alpha n_0, n_a = (-alpha, 0, 0, 0)
+  const T anC = M.alpha * nC;
 #pragma unroll 1
-    for (int s = 0; s < 10; ++s) {
-      const int a = s < 4 ? 0 : (s < 7 ? 1 : (s < 9 ? 2 : 3));
-      const int b = s - (a == 0 ? 0 : (a == 1 ? 3 : (a == 2 ? 5 : 6)));
-      // d_a H_b: rows (x, b) = 4 x + b of dH for a = x + 1; d_t H_b is row
-      // 12 + b when the gauge source is evolved with its time derivative
-      // (58 fields), else zero
+  for (int b = 0; b < 4; ++b) {
+    const SymRow rb(b);
+    T Gce[10];  // Gamma_b^{ce}, symmetric, off-diagonal weight 2
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      T Gcf[4];  // Gamma_b^c_f = g^cd Gamma_bdf
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        Acc<T> acc;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) acc.fma_(M.gi4[SI(c, d)], V(b * 10 + SI(d, f)));
+        Gcf[f] = acc.get();
+      }
+#pragma unroll
+      for (int e = c; e < 4; ++e) {
+        Acc<T> acc;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc.fma_(M.gi4[SI(e, f)], Gcf[f]);
+        Gce[SI(c, e)] = (c == e) ? acc.get() : twice(acc.get());
+      }
+    }
+#pragma unroll 1
+    for (int a = 0; a <= b; ++a) {
+      const int s = rb(a);
+      // S_Pi = -2 alpha nabla_(a H_b) + alpha (n_b C_a + n_a C_b - g_ab n^c C_c);
+      // d_a H_b: rows (x, b) = 4 x + b of dH for a = x + 1; d_t H_b is row 12 + b
+      // when the gauge source is evolved with its time derivative (58 fields),
+      // else zero
       const T dHab = a == 0 ? (dtH ? ldA<T, kInt<T>>(dH, P, p, 12 + b) : zero)
                             : ldA<T, kInt<T>>(dH, P, p, (a - 1) * 4 + b);
       const T dHba = b == 0 ? (dtH ? ldA<T, kInt<T>>(dH, P, p, 12 + a) : zero)
                             : ldA<T, kInt<T>>(dH, P, p, (b - 1) * 4 + a);
+      const T gab = ldA<T, FU>(u, P, p, s);
+      // -2 alpha g^cd g^ef Gamma_ace Gamma_bdf
+      Acc<T> qa;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int e = c; e < 4; ++e) qa.fma_(V(a * 10 + SI(c, e)), Gce[SI(c, e)]);
       Acc<T> acc;
       acc.add(half_of(dHab + dHba));
 #pragma unroll
@@ -193,57 +221,15 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
       const T DH = acc.get();
       Acc<T> v;
       v.fma_(-twoal, DH);
-      v.fma_(-(anC), ldA<T, FU>(u, P, p, s));
-      if (a == 0) v.fma_(aa, V(50 + b));
-      if (b == 0) v.fma_(aa, V(50 + a));
-      V(40 + s) = v.get();
+      v.fma_(-(anC), gab);
+      if (a == 0) v.fma_(aa, V(40 + b));
+      if (b == 0) v.fma_(aa, V(40 + a));
+      Acc<T> r;
+      r.add(v.get());
+      r.fma_(m2al, qa.get());
+      stA<T, kInt<T>>(src, P, p, s, r.get());
     }
   }
-  // -2 alpha g^cd g^ef Gamma_ace Gamma_bdf
-  {
-    const T m2al = -(M.alpha + M.alpha);
-#pragma unroll 1
-    for (int b = 0; b < 4; ++b) {
-      const SymRow rb(b);
-      T Gce[10];  // Gamma_b^{ce}, symmetric, off-diagonal weight 2
-      {
-        T Gcf[4][4];  // Gamma_b^c_f = g^cd Gamma_bdf
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-          for (int f = 0; f < 4; ++f) {
-            Acc<T> acc;
-#pragma unroll
-            for (int d = 0; d < 4; ++d) acc.fma_(M.gi4[SI(c, d)], V(b * 10 + SI(d, f)));
-            Gcf[c][f] = acc.get();
-          }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-          for (int e = c; e < 4; ++e) {
-            Acc<T> acc;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) acc.fma_(M.gi4[SI(e, f)], Gcf[c][f]);
-            Gce[SI(c, e)] = (c == e) ? acc.get() : twice(acc.get());
-          }
-      }
-#pragma unroll 1
-      for (int a = 0; a <= b; ++a) {
-        Acc<T> qa;
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-          for (int e = c; e < 4; ++e) qa.fma_(V(a * 10 + SI(c, e)), Gce[SI(c, e)]);
-        Acc<T> acc;
-        const int s = 40 + rb(a);
-        acc.add(V(s));
-        acc.fma_(m2al, qa.get());
-        V(s) = acc.get();
-      }
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < 10; ++s) stA<T, kInt<T>>(src, P, p, s, V(40 + s));
 }
 
 // The Phi-Phi and Pi-Pi terms of eq. Pidot and the remaining algebraic terms
