@@ -604,13 +604,13 @@ static int filter_in_step(cffyn_shell* sh, double* spin, cudaStream_t st, Run&& 
 }
 
 // conc: the algebraic right-hand-side kernels (k_rhs_gamma, k_rhs_quad: they
-// read the stage state only) run on the shell's second stream beside the
-// d_theta + d_phi launch, which they share no buffer with, and join before
-// the principal parts; forked after d_r (forked at the start of the stage,
-// they held up the exponent scan and d_r: 3.233 vs 3.248 ms per step), but at
-// the start for small shells, whose launches leave SMs idle; not
-// for the evolved gauge of 54/58 fields (k_gauge_rhs reads the derivatives)
-// nor under per-group timing.
+// read the stage state only) run on the shell's second stream beside the exponent
+// scan and the derivative launches, which they share no buffer with, and join
+// before the principal parts.  Forked at the stage's start: forked after d_r they
+// end after the derivatives (RK4 step, us: 25 x 28 x 56 points 1016 against 881, 33
+// x 48 x 96 2493 against 2408, 49 x 56 x 112 5715 either way; eight shells in a batch
+// 12.85 against 12.23 ms).  Not for the evolved gauge of 54/58 fields
+// (k_gauge_rhs reads the derivatives) nor under per-group timing.
 template <class Run>
 static int stage_front(cffyn_shell* sh, double* u, int s, cudaStream_t st, Run&& run, bool conc) {
   const size_t nvP = (size_t)sh->nv * P_all(sh);
@@ -620,29 +620,25 @@ static int stage_front(cffyn_shell* sh, double* u, int s, cudaStream_t st, Run&&
   const double* X = stage_state_of(sh, u, s);
   int rc;
   const bool fork = conc && sh->ng == 0 && sh->aux_stream;
-  const bool early = fork && pw_rhs_shared(sh);
-  cudaStream_t sa = fork ? sh->aux_stream : st;
-  auto algebraic = [&]() -> int {
+  auto algebraic = [&](cudaStream_t sa) -> int {
     int r;
-    CF_CUDA(cudaEventRecord(sh->ev_fork, st));
-    CF_CUDA(cudaStreamWaitEvent(sa, sh->ev_fork, 0));
     if ((r = run(2, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 1, xp, true, sa); }))) return r;
-    if ((r = run(3, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 2, xp, true, sa); }))) return r;
-    CF_CUDA(cudaEventRecord(sh->ev_join, sa));
-    return CFFYN_OK;
+    return run(3, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 2, xp, true, sa); });
   };
-  if (early && (rc = algebraic())) return rc;
+  if (fork) {
+    CF_CUDA(cudaEventRecord(sh->ev_fork, st));
+    CF_CUDA(cudaStreamWaitEvent(sh->aux_stream, sh->ev_fork, 0));
+    if ((rc = algebraic(sh->aux_stream))) return rc;
+    CF_CUDA(cudaEventRecord(sh->ev_join, sh->aux_stream));
+  }
   if ((rc = run(10, [&] { return op_prepare(sh, X, xp, nf, P, 0, st); }))) return rc;
   if ((rc = run(0, [&] { return op_deriv_r(sh, X, sh->D, nf, xp, st); }))) return rc;
-  if (fork && !early && (rc = algebraic())) return rc;
   if ((rc = run(1, [&] { return op_deriv_theta_phi(sh, X, sh->D + nvP, sh->D + 2 * nvP, nf, xp, st); })))
     return rc;
-  if (fork) {
+  if (fork)
     CF_CUDA(cudaStreamWaitEvent(st, sh->ev_join, 0));
-  } else {
-    if ((rc = run(2, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 1, xp, true, st); }))) return rc;
-    if ((rc = run(3, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 2, xp, true, st); }))) return rc;
-  }
+  else if ((rc = algebraic(st)))
+    return rc;
   return run(4, [&] { return pw_rhs_part(sh, X, sh->D, sh->S, 3, xp, true, st); });
 }
 

@@ -902,15 +902,17 @@ __global__ void __launch_bounds__(128) k_gauge_rhs(const double* __restrict__ u,
   }
 }
 
-// Whether a point's tensors are shared out over four warps: up to one wave of the
-// one-point-per-thread blocks (four per SM; gamma / quad, us, one thread against
-// four warps per point: 2106 points 30 / 25 against 11 / 10, 39168 points 37 / 38
-// against 29 / 35, 102400 points 69 / 72 against 69 / 74, 152064 points 81 / 91
-// against 97 / 106).
+// Whether a point's tensors are shared out over four warps: up to 2.5 blocks of
+// one point per thread per SM.  gamma / quad, us, one thread against four warps per
+// point: 2106 points 14.7 / 13.7 against 8.9 / 7.9, 11250 points 15.5 / 14.0 against
+// 10.5 / 9.8, 28800 points 21.1 / 17.8 against 22.0 / 16.9, 67584 points 32.4 / 31.8
+// against 39.7 / 35.4.  The line lies above where the two meet because the call
+// of an FP64 state goes without its pair copy below it (right-hand side, us: 28800
+// points 132 against 119, 39200 points 167 against 163, 67584 points 216 against 233).
 // Blocks of a batch's other classes count too: beside them the shorter chain buys
 // nothing and the repeated work costs (batch of eight shells 14.7 against 15.4 ms).
 static bool rhs_shared(const cffyn_shell* sh, unsigned nbr) {
-  return nbr + sh->beside / kRhsBlock <= 4ll * sh->sm_count;
+  return 2 * (nbr + sh->beside / kRhsBlock) <= 5ll * sh->sm_count;
 }
 bool pw_rhs_shared(const cffyn_shell* sh) { return rhs_shared(sh, blocks_for((long long)P_all(sh), kRhsBlock)); }
 
