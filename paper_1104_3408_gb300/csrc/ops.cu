@@ -11,13 +11,13 @@
 // Two arithmetic cores share the column descriptors and the gathers:
 //   FP64   plain double FMA on CUDA cores (k_op_fp64, the reference path);
 //   MIXED  split-precision products on the fifth-generation tensor cores
-//          (k_op_tc): W and each input column are written as 47-bit
-//          fixed-point integers relative to a per-row / per-field power of two
-//          and cut into six balanced 8-bit digits held exactly in BF16; digit
-//          products are summed by tcgen05.mma in FP32 accumulators in tensor
-//          memory (see the k_op_tc comment for the exactness argument); pairs
-//          with i + j > 5 are dropped (relative truncation about 6 * 2^-48 of
-//          |W| |x| K).
+//          (k_op_ws, and k_op_tc for small launches): W and each input column
+//          are written as 47-bit fixed-point integers relative to a per-row /
+//          per-field power of two and cut into six balanced 8-bit digits held
+//          exactly in BF16; digit products are summed by tcgen05.mma in FP32
+//          accumulators in tensor memory (see the k_op_ws comment for the
+//          exactness argument); pairs with i + j > 6 (the filter's operators: > 5)
+//          are dropped.
 #include <algorithm>
 #include <cstdio>
 
@@ -758,7 +758,7 @@ __device__ __forceinline__ int col_exponent(const TcBatch& B, const OpArgs& a, c
 // columns.  2 (ROWS = 48, odd n_r up to kRawRows): also the inputs come as one bulk
 // copy per tile, into one of two buffers that the tile's outputs then take (each
 // thread's 16 words of a line, 8 bytes per load and a line apart across the
-// lanes, were 32 sectors per load: 61 against 38 us for 50 fields of 33 x 48 x 96;
+// lanes, were 32 sectors per load: 61 against 56 us for 50 fields of 33 x 48 x 96;
 // odd, so that the lanes' words lie in different banks).
 constexpr int kRawRows = 39;
 template <bool FI, int ROWS, int STAGE>
@@ -1332,12 +1332,18 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads)
 
 static int tiles_of(const OpArgs& a) { return (int)((a.g.ncols + kTcCols - 1) / kTcCols); }
 
-// Whether a launch of so many items takes the persistent kernel.  It pays from
-// a few items per SM on: with 96 rows (the one-item kernel holds one CTA per
-// SM) 297 / 322 / 1238 items take 27 / 35 / 96 us against 31 / 43 / 133; with 48
-// (two per SM) 470 items of d_theta + d_phi 24.3 against 25.7 us, 846 / 1128 items
-// of the projection 33 / 38 against 43 / 57, 1800 of d_r 57 against 65, but 450 of
-// d_r 19.6 against 17.4.
+// Whether a launch of so many items takes the persistent kernel.  With 96 rows
+// (the one-item kernel holds one CTA per SM) it pays from more than one item per SM
+// on: 297 / 322 / 1238 items take 27 / 35 / 96 us against 31 / 43 / 133 when it came in, an
+// RK4 step of 33 x 32 x 64 takes 1204 us, 1242 with the line at two.  With 48 rows (two
+// CTAs per SM) it pays by itself from some two items per SM on (470 items of d_theta
+// + d_phi 24.3 against 25.7 us, 846 / 1128 of the projection 33 / 38 against 43 / 57, 1800
+// of d_r 57 against 65, but 450 of d_r 19.6 against 17.4), but it holds the SMs
+// that the algebraic kernels and the filter's second chain run on beside it: RK4
+// steps with the line at 2, 3, 5, 8 per SM, us: 25 x 28 x 56 points 893 / 894 / 882 /
+// 884, 17 x 48 x 96 points 1444 / 1443 / 1471 / 1471, 33 x 32 x 64 points 1204 / 1204 / 1204 /
+// 1220, 33 x 40 x 80 points 1789 / 1789 / 1788 / 1813; five, so that no size is slower than
+// with the one-item kernel.
 static bool runs_persistent(const cffyn_shell* sh, int rows, long long items) {
   return items > (rows == 48 ? 5 : 1) * (long long)sh->sm_count;
 }

@@ -1,11 +1,6 @@
 // Pointwise kernels of the hot path, templated on the arithmetic type
 // (double for the FP64 path, ff = FP32 pair for the mixed path):
 //
-//   k_rhs          Cartesian derivatives by the chain rule (eq. dvdx), the
-//                  first-order GHG right-hand side (App. A.1 eqs. gdot, Phidot,
-//                  Pidot, dependent quantities from eqs. normal, abgfromgab,
-//                  Gamma) and the freeze-incoming boundary condition on the
-//                  outermost sphere (App. A.2, B = E^-1 Z E).
 //   k_decompose    Cartesian tensor groups -> spin-weighted components
 //                  (Sec. 3.4, eq. tensorexpansion) written as real multiples of
 //                  the triad components: every tensor is first rotated to the
@@ -577,7 +572,9 @@ __device__ __forceinline__ void reconstruct_update(Scratch<T> sc, const double* 
 // Latency-bound (a few dependent loads and stores per field): nine blocks
 // per SM, i.e. at most 56 registers and 18 KB of slots per block (with 80
 // registers and 36 slots, six blocks: 0.423 ms per step on the 33 x 48 x 96
-// shell; eight blocks, 64 registers: 0.340; nine: 0.335, same results).
+// shell; eight blocks, 64 registers: 0.340; nine: 0.335, same results).  By now 64
+// us per launch of stages 1-3 (365 MB, 54 us at the copy bandwidth) and 90 of the
+// last stage.
 template <class T, bool FD, int KIND>
 __global__ void __launch_bounds__(128, 9) k_reconstruct(const double* __restrict__ sp, double* __restrict__ dst,
                                                      Geo geo, int mode, double* __restrict__ u,
@@ -609,9 +606,9 @@ __global__ void __launch_bounds__(128, 9) k_reconstruct(const double* __restrict
 // ---------------------------------------------------------------------------
 // k_reconstruct for few points (recon_shared): 32 points per block with eight
 // warps, each warp a share of every point's tensor components.  As one thread
-// per tensor group the rank-3 group's 18 components are one chain of 14 us
-// (stages 1-3) to 31 us (last stage) however few points there are; shared out it
-// takes 9 to 17 (13 x 9 x 18).  The three warps of the rank-3 tensor exchange
+// per tensor group the rank-3 group's 18 components are one chain of 12 us
+// (stages 1-3) to 18 us (last stage) however few points there are; shared out it
+// takes 9 to 14 (13 x 9 x 18).  The three warps of the rank-3 tensor exchange
 // their legs through shared memory, [slot][point].  Same results.
 //
 // Shares: 0..2 the legs of group 7 (six components each), 3 group 6 (nine), 4 and
@@ -852,8 +849,8 @@ __global__ void __launch_bounds__(32 * kShares, 4)
 // One thread per point and share of the fields (blockIdx.y, cart_split): the
 // Jacobian is formed once from the tables and applied to every field of the
 // share, whose values are coalesced across the threads.  Bound by the FP64 pipe
-// (eight operations per value at 0.49 T/s: 55 us for 50 fields of 33 x 32 x 64);
-// with all fields in one thread and the divisions in the kernel 118 us.
+// (eight operations per value at 0.49 T/s: 55 us of the 72 for 50 fields of 33 x 32
+// x 64); with all fields in one thread and the divisions in the kernel 118 us.
 // status (may be NULL): a status word of the operator launches that produced
 // D; if it is non-zero (a timed-out wait) every output value is a NaN.
 template <bool FI, bool FO>
@@ -1013,8 +1010,9 @@ int pw_decompose(const cffyn_shell* sh, const double* in, double* out, bool in_p
 }
 
 // Whether a point's components are shared out over eight warps: up to one block of
-// 128 points per SM (stages 1-3 / last stage, us: 8704 points 15 / 24 against 31 /
-// 38, 28800 points 27 / 45 against 31 / 41, 152064 points 110 / 177 against 71 / 101).
+// 128 points per SM (stages 1-3 / last stage, us, against one thread per tensor
+// group: 8704 points 11 / 18 and 12 / 19, 11250 points 12 / 20 and 14 / 22, 28800 points
+// 27 / 42 and 27 / 36, 67584 points 52 / 79 and 33 / 47).
 static bool recon_shared(const cffyn_shell* sh, unsigned nb) { return nb + sh->beside / 128 <= sh->sm_count; }
 
 // dst (mode 0) is an FP64 array; uf (mixed path): the step's initial state as

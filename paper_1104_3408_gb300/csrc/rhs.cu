@@ -81,8 +81,13 @@ constexpr int kRhsBlock = 128;
 constexpr int kGamSlots = 44;   // Gamma_cab (c*10 + s) | C_a 40..43
 constexpr int kQuadSlots = 40;  // Pi 0..9 | Phi_iab 10 + 10 i + s
 
-// Four blocks per SM: 128 registers, 54 KB of slots (g_ab is read again from
-// u where the gauge terms need it instead of holding ten more slots).
+// Bound by instruction issue (two thirds of the slots; 10750 instructions per
+// point, most of them the pair sums).  Four blocks per SM: 128 registers, 44 KB of
+// slots (five blocks of 96 registers: 72 against 67 us for 33 x 48 x 96 points);
+// g_ab is read again from u where the gauge terms need it.  A pair's gauge terms
+// are formed where its quadratic term is: in a loop of their own they waited for
+// their words (71 us).  81 us before that and the shorter pair sums (Acc, half_of,
+// gamma_cab).
 template <class T, bool FU, bool FO>
 __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __restrict__ u,
                                                          const double* __restrict__ H,
@@ -234,6 +239,10 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_gamma(const double* __rest
 
 // The Phi-Phi and Pi-Pi terms of eq. Pidot and the remaining algebraic terms
 // of eqs. Pidot and Phidot; alpha, beta^i, gamma^ij come from k_rhs_gamma.
+// Bound by instruction issue (11660 per point); 33 x 48 x 96 points: 66 us, with each
+// pair's quadratic terms kept in ten more slots for a second loop 69, with the
+// selects of SI in the rolled loops 86 (see SymRow), with n^c n^d A_cd from sixteen
+// products 74; five blocks per SM (96 registers) 75.
 template <class T, bool FU>
 __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_quad(const double* __restrict__ u, double* __restrict__ src,
                                                         Geo geo) {
@@ -371,8 +380,8 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_quad(const double* __restr
 // k_rhs_gamma and k_rhs_quad for few points (rhs_shared): 32 points per block and
 // four warps, each warp a share of every point's tensors.  One thread's chain
 // through a whole point takes 30 and 25 us however few points there are; shared
-// out it takes 11 and 10 (13 x 9 x 18), at the price of barriers and repeated
-// 3+1 quantities.  The tensors live in shared memory as [slot][point], written by
+// out it takes 11 and 10 (13 x 9 x 18; by now 15 and 14 against 9 and 8), at the
+// price of barriers and repeated 3+1 quantities.  The tensors live in shared memory as [slot][point], written by
 // one warp and read by all.  Every sum runs in the order of the kernels above:
 // the results are bit-identical.
 template <class T>
@@ -722,7 +731,8 @@ __device__ __forceinline__ void copies_pending_at_most() {
 
 // The words of a symmetric pair (15 derivatives, 4 sources) are copied to shared
 // memory one pair ahead: held in registers only one pair's loads were in flight
-// (DRAM 54 %, half the warps' time waiting for them).
+// (DRAM 54 %, half the warps' time waiting for them).  Now 52 us for 33 x 48 x 96
+// points, 292 MB at 83 % of the copy bandwidth.
 constexpr int kPpWords = 19;
 
 // blockIdx.y: the block's share of the ten symmetric pairs (pp_split).
@@ -918,7 +928,7 @@ bool pw_rhs_shared(const cffyn_shell* sh) { return rhs_shared(sh, blocks_for((lo
 
 // Shares of the ten symmetric pairs per point in k_rhs_pp: one thread's loop over
 // all ten takes 27 us by itself (its loads wait one after the other), in ten
-// shares 9.5 (13 x 9 x 18); every share repeats the chain-rule coefficients, so
+// shares 9.5, with the words copied ahead 6 (13 x 9 x 18); every share repeats the chain-rule coefficients, so
 // only as many are taken as fill one wave (four blocks per SM).
 static unsigned pp_split(const cffyn_shell* sh, unsigned nb) {
   for (unsigned n : {10u, 5u, 2u})
@@ -999,7 +1009,7 @@ int pw_rhs_part(const cffyn_shell* sh, const double* u, const double* D, double*
 // Right-hand side of an FP64 state into an FP64 array.  On the mixed path large
 // launches read the state from a pair copy in Uf (the step calls fill it anew):
 // converted once instead of by every kernel that reads it (gamma and quad of
-// 33 x 48 x 96: 142 + 130 us, with the copy 28 + 81 + 91).
+// 33 x 48 x 96: 142 + 130 us, with the copy 28 + 81 + 91 then, 18.5 + 67 + 66 now).
 int pw_rhs(const cffyn_shell* sh, const double* u, const double* D, double* out, cudaStream_t st) {
   if (sh->d.precision != CFFYN_MIXED || pw_rhs_shared(sh)) return pw_rhs_part(sh, u, D, out, 0, false, false, st);
   const int rc = pw_to_internal(sh, u, sh->Uf, (long long)sh->nv * (long long)sh->P, st);
