@@ -573,8 +573,9 @@ __device__ __forceinline__ void reconstruct_update(Scratch<T> sc, const double* 
 // per SM, i.e. at most 56 registers and 18 KB of slots per block (with 80
 // registers and 36 slots, six blocks: 0.423 ms per step on the 33 x 48 x 96
 // shell; eight blocks, 64 registers: 0.340; nine: 0.335, same results).  By now 64
-// us per launch of stages 1-3 (365 MB, 54 us at the copy bandwidth) and 90 of the
-// last stage.
+// us per launch of stages 1-3 (304 MB, 45 us at the copy bandwidth; issue 0.63 per
+// scheduler and cycle, waits for loads and for instructions) and 90 of the last
+// stage.
 template <class T, bool FD, int KIND>
 __global__ void __launch_bounds__(128, 9) k_reconstruct(const double* __restrict__ sp, double* __restrict__ dst,
                                                      Geo geo, int mode, double* __restrict__ u,
