@@ -1336,16 +1336,16 @@ static int tiles_of(const OpArgs& a) { return (int)((a.g.ncols + kTcCols - 1) / 
 // (the one-item kernel holds one CTA per SM) it pays from more than one item per SM
 // on: 297 / 322 / 1238 items take 27 / 35 / 96 us against 31 / 43 / 133 when it came in, an
 // RK4 step of 33 x 32 x 64 takes 1204 us, 1242 with the line at two.  With 48 rows (two
-// CTAs per SM) it pays by itself from some two items per SM on (470 items of d_theta
-// + d_phi 24.3 against 25.7 us, 846 / 1128 of the projection 33 / 38 against 43 / 57, 1800
-// of d_r 57 against 65, but 450 of d_r 19.6 against 17.4), but it holds the SMs
-// that the algebraic kernels and the filter's second chain run on beside it: RK4
-// steps with the line at 2, 3, 5, 8 per SM, us: 25 x 28 x 56 points 893 / 894 / 882 /
-// 884, 17 x 48 x 96 points 1444 / 1443 / 1471 / 1471, 33 x 32 x 64 points 1204 / 1204 / 1204 /
-// 1220, 33 x 40 x 80 points 1789 / 1789 / 1788 / 1813; five, so that no size is slower than
-// with the one-item kernel.
-static bool runs_persistent(const cffyn_shell* sh, int rows, long long items) {
-  return items > (rows == 48 ? 5 : 1) * (long long)sh->sm_count;
+// CTAs per SM) it pays by itself from two to three items per SM on (470 items of
+// d_theta + d_phi 24.3 against 25.7 us, 846 / 1128 of the projection 33 / 38 against 43 /
+// 57), later for d_r (dr; three k-steps at most: 450 items 19.6 against 17.4, 1800 items 57
+// against 65), but it holds the SMs that the algebraic kernels and the filter's
+// second chain run on beside it.  Lines at 2, 3, 4, 5 items per SM (d_r at 5), RK4 step,
+// us: 25 x 20 x 40 points 545 / 541 / 542 / 541, 33 x 24 x 48 points 797 / 787 / 786 / 794, 17 x
+// 48 x 96 points 1449 / 1449 / 1448 / 1476, right-hand side of 25 x 24 x 48 points 113 / 113 /
+// 119 / 119; d_r at 3: 25 x 28 x 56 points 894 against 882.
+static bool runs_persistent(const cffyn_shell* sh, int rows, long long items, bool dr = false) {
+  return items > (rows != 48 ? 1 : dr ? 5 : 3) * (long long)sh->sm_count;
 }
 
 // Mixed path: one launch of the tcgen05 core over the classes of b (same row
@@ -1369,7 +1369,7 @@ static int launch_batch(const cffyn_shell* sh, const TcBatch& b0, cudaStream_t s
   const int rows = b.W[0].rows;
   // d_r (one class, one row group): the instance with the staged epilogue
   const bool dr = b.nclass == 1 && b.a[0].kind == OP_R && b.W[0].ngroups == 1;
-  const bool persistent = runs_persistent(sh, rows, items);
+  const bool persistent = runs_persistent(sh, rows, items, dr);
   const int P = b.a[0].g.P, out_bytes = kTcCols * P * (int)sizeof(double);
   // d_r's tiles beside the persistent kernel's ring
   const int ring = rows == 48 ? WsCfg<48>::kStage * kRingStages<48, 1> : WsCfg<96>::kStage * kRingStages<96, 1>;
