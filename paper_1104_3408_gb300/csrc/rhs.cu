@@ -719,8 +719,9 @@ __global__ void __launch_bounds__(kRhsBlock)
 }
 
 // Asynchronous copy of one 8-byte word to shared memory (the thread's own word:
-// it waits for its own copies, no barrier).
-__device__ __forceinline__ void copy8_async(void* dst, const double* src) {
+// it waits for its own copies, no barrier).  Both addresses must be 8-byte aligned:
+// the destination's type sees to it (a pair of floats alone is aligned to 4).
+__device__ __forceinline__ void copy8_async(unsigned long long* dst, const double* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned int)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
@@ -735,11 +736,21 @@ __device__ __forceinline__ void copies_pending_at_most() {
 // points, 292 MB at 83 % of the copy bandwidth.
 constexpr int kPpWords = 19;
 
+// value of a copied word of internal storage
+template <class T> __device__ __forceinline__ T word_value(unsigned long long w);
+template <> __device__ __forceinline__ double word_value<double>(unsigned long long w) {
+  return __longlong_as_double((long long)w);
+}
+template <> __device__ __forceinline__ ff word_value<ff>(unsigned long long w) {
+  return ff{__uint_as_float((unsigned int)w), __uint_as_float((unsigned int)(w >> 32))};
+}
+
 // blockIdx.y: the block's share of the ten symmetric pairs (pp_split).
 template <class T, bool FO>
 __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, const double* __restrict__ src,
                                                 double* __restrict__ out, Geo geo) {
-  __shared__ T buf[2][kPpWords][128];
+  __shared__ unsigned long long buf[2][kPpWords][128];
+  static_assert(alignof(decltype(buf)) == 8, "8-byte copies");
   const long long P = geo.P;
   const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (p >= P) return;
@@ -750,7 +761,7 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
   // words 5 m .. 5 m + 4: d_m of g_s, Pi_s, Phi_xs; 15: source of d_t Pi_s, 16..18:
   // of d_t Phi_xs
   auto fetch = [&](int s) {
-    T(*w)[128] = buf[(s - s0) & 1];
+    unsigned long long(*w)[128] = buf[(s - s0) & 1];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       const double* d = D + (long long)m * nv * P + p;
@@ -824,7 +835,7 @@ __global__ void __launch_bounds__(128) k_rhs_pp(const double* __restrict__ D, co
     } else {
       copies_pending_at_most<0>();
     }
-    auto word = [&](int e) -> T { return buf[(s - s0) & 1][e][threadIdx.x]; };
+    auto word = [&](int e) -> T { return word_value<T>(buf[(s - s0) & 1][e][threadIdx.x]); };
     T Dd[3], DPh[3][3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
