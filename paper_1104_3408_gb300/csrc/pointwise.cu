@@ -743,12 +743,14 @@ struct StageUpdate {
   __device__ __forceinline__ StateWords<T, KIND> fetch(int f) const {
     const long long o = (long long)f * P + p;
     StateWords<T, KIND> x;
+    // a spare thread reads words that this kernel does not write in place of those
+    // that the last point's own thread is writing (no branch; the values go unused)
     if (KIND == 1) {
       // stage state: FP64 sum on the FP64 path, double-float on the mixed path
       x.base = kPair ? SI_::ld(uf, o) : S<T>::c(__ldg(u + o));
-      if (stage != 0) x.acc = SI_::ld(kacc, o);
+      if (stage != 0) x.acc = SI_::ld(live ? kacc : kPair ? uf : u, o);
     } else if (KIND == 2) {
-      x.un = __ldg(u + o);
+      x.un = __ldg((live ? u : kacc) + o);
       x.acc = SI_::ld(kacc, o);
     }
     return x;

@@ -672,7 +672,8 @@ __global__ void __launch_bounds__(kRhsBlock)
     for (int a = 0; a <= b; ++a) {
       const SymRow ra(a);
       const int s = rb(a);
-      const T part = ldA<T, kInt<T>>(src, P, p, s);
+      // (a spare thread reads alpha: word s is being written by the last point's own)
+      const T part = ldA<T, kInt<T>>(src, P, p, live ? s : 40);
       Acc<T> q2;
 #pragma unroll
       for (int c = 0; c < 4; ++c) q2.fma_(-V(kQPi + ra(c)), Piu[c]);
