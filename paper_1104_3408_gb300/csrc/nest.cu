@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(128) k_interface(const double* __restrict__ XA
   const T half = S<T>::c(0.5);
 #pragma unroll 1
   for (int c = 0; c < 10; ++c) {
-    auto lda = [&](int f) { return Store<T, FR>::ld(SA, (long long)f * PA + pa); };
-    auto ldb = [&](int f) { return Store<T, FR>::ld(SB, (long long)f * PB + pb); };
+    auto lda = [&](int f) { return Store<T, FR>::ld_rw(SA, (long long)f * PA + pa); };
+    auto ldb = [&](int f) { return Store<T, FR>::ld_rw(SB, (long long)f * PB + pb); };
     const T ag = lda(c), aPi = lda(10 + c), bg = ldb(c), bPi = ldb(10 + c);
     T aPh[3], bPh[3];
 #pragma unroll
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(128) k_interface(const double* __restrict__ XA
     }
   }
   for (int f = 50; f < ga.nv; ++f)
-    Store<T, FR>::st(SB, (long long)f * PB + pb, Store<T, FR>::ld(SA, (long long)f * PA + pa));
+    Store<T, FR>::st(SB, (long long)f * PB + pb, Store<T, FR>::ld_rw(SA, (long long)f * PA + pa));
 }
 
 // Coupling on the common sphere of shells a (inner) and b (outer): XA the

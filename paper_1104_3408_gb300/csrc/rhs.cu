@@ -32,6 +32,11 @@ template <class T, bool F>
 __device__ __forceinline__ T ldA(const double* a, long long P, long long p, int f) {
   return Store<T, F>::ld(a, (long long)f * P + p);
 }
+// of an array that the kernel also writes (see Store)
+template <class T, bool F>
+__device__ __forceinline__ T ldA_rw(const double* a, long long P, long long p, int f) {
+  return Store<T, F>::ld_rw(a, (long long)f * P + p);
+}
 template <class T, bool F>
 __device__ __forceinline__ void stA(double* a, long long P, long long p, int f, T v) {
   Store<T, F>::st(a, (long long)f * P + p, v);
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(kRhsBlock, 4) k_rhs_quad(const double* __restr
 #pragma unroll
           for (int c = 0; c < 4; ++c) q.fma_(V(10 + 10 * x + ra(c)), W[x][c]);
         Acc<T> acc;
-        acc.add(ldA<T, kInt<T>>(src, P, p, s));
+        acc.add(ldA_rw<T, kInt<T>>(src, P, p, s));
         acc.fma_(twoal, q.get());
         acc.fma_(cPi, V(s));
 #pragma unroll
@@ -673,7 +678,7 @@ __global__ void __launch_bounds__(kRhsBlock)
       const SymRow ra(a);
       const int s = rb(a);
       // (a spare thread reads alpha: word s is being written by the last point's own)
-      const T part = ldA<T, kInt<T>>(src, P, p, live ? s : 40);
+      const T part = ldA_rw<T, kInt<T>>(src, P, p, live ? s : 40);
       Acc<T> q2;
 #pragma unroll
       for (int c = 0; c < 4; ++c) q2.fma_(-V(kQPi + ra(c)), Piu[c]);

@@ -257,19 +257,36 @@ template <> struct S<ff> {
 // as float2 (FF = true); both are 8 bytes per value.  Internal buffers of the
 // mixed path use the pair form, so that its pointwise kernels load and store
 // without any conversion.
+//
+// ld is for arrays that the launch only reads (the read-only path may hold a word
+// for the whole launch).  A word that the launch also writes is read with ld_rw, an
+// ordinary load; its asm is neither volatile nor clobbers memory, as the thread's one
+// store to that word takes the loaded value.
+__device__ __forceinline__ double load_rw(const double* a) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(a));
+  return v;
+}
 template <class T, bool FF> struct Store;
 template <> struct Store<double, false> {
   static __device__ __forceinline__ double ld(const double* b, long long i) { return b[i]; }
+  static __device__ __forceinline__ double ld_rw(const double* b, long long i) { return load_rw(b + i); }
   static __device__ __forceinline__ void st(double* b, long long i, double v) { b[i] = v; }
 };
 template <> struct Store<ff, false> {
   static __device__ __forceinline__ ff ld(const double* b, long long i) { return ff_from_double(__ldg(b + i)); }
+  static __device__ __forceinline__ ff ld_rw(const double* b, long long i) { return ff_from_double(load_rw(b + i)); }
   static __device__ __forceinline__ void st(double* b, long long i, ff v) { b[i] = ff_to_double(v); }
 };
 template <> struct Store<ff, true> {
   static __device__ __forceinline__ ff ld(const double* b, long long i) {
     const float2 v = __ldg(reinterpret_cast<const float2*>(b) + i);
     return ff{v.x, v.y};
+  }
+  static __device__ __forceinline__ ff ld_rw(const double* b, long long i) {
+    ff v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.hi), "=f"(v.lo) : "l"(b + i));
+    return v;
   }
   static __device__ __forceinline__ void st(double* b, long long i, ff v) {
     reinterpret_cast<float2*>(b)[i] = make_float2(v.hi, v.lo);

@@ -3,6 +3,9 @@ write in the same array.  The last block's spare threads repeat the last point
 without storing anything: they must not read the words that this point's own
 threads are storing.
 
+Words that a launch also writes are read with ordinary loads, not through the
+read-only path.
+
 The update of k_reconstruct_shared (StageUpdate) runs here on the host, compiled
 from its source text against stand-ins that count every read."""
 
@@ -20,11 +23,12 @@ _HARNESS = r"""
 #include <vector>
 #define __device__
 #define __forceinline__ inline
-static std::vector<const double*> reads;
-static double __ldg(const double* p) { reads.push_back(p); return *p; }
+static std::vector<const double*> reads, cached;  // all reads; those through the read-only path
+static double __ldg(const double* p) { reads.push_back(p); cached.push_back(p); return *p; }
 template <class T> struct S { static T c(double x) { return x; } static double to_double(T x) { return x; } };
 template <class T, bool F> struct Store {
-  static T ld(const double* b, long long i) { reads.push_back(b + i); return b[i]; }
+  static T ld(const double* b, long long i) { return __ldg(b + i); }
+  static T ld_rw(const double* b, long long i) { reads.push_back(b + i); return b[i]; }
   static void st(double* b, long long i, T v) { b[i] = v; }
 };
 template <class T> constexpr bool kIn = PAIRS;
@@ -36,12 +40,17 @@ template <int KIND> void run(bool live) {
   for (int i = 0; i < 8; ++i) u[i] = k[i] = uf[i] = i + 1;
   StageUpdate<double, KIND> up{dst, u, U, k, uf, 4, 3, KIND == 2 ? 3 : 1, live, false, 0.5, 0.25};
   reads.clear();
+  cached.clear();
   up.put(1, 10.0, up.fetch(1));
   // reads of arrays that this kind of update writes
-  int r = 0;
-  for (const double* p : reads)
-    for (const double* a : {KIND == 1 ? k : u, KIND == 1 ? U : uf}) r += p >= a && p < a + 8;
-  std::printf("%%d %%d %%g %%g %%g %%g %%g\n", KIND, r, dst[7], u[7], U[7], k[7], uf[7]);
+  auto written = [&](const std::vector<const double*>& v) {
+    int n = 0;
+    for (const double* p : v)
+      for (const double* a : {KIND == 1 ? k : u, KIND == 1 ? U : uf}) n += p >= a && p < a + 8;
+    return n;
+  };
+  const int r = written(reads), c = written(cached);
+  std::printf("%%d %%d %%g %%g %%g %%g %%g\n", c, r, dst[7], u[7], U[7], k[7], uf[7]);
 }
 int main() { run<0>(true); run<1>(true); run<2>(true); run<0>(false); run<1>(false); run<2>(false); }
 """
@@ -74,6 +83,7 @@ def test_spare_threads_read_no_word_that_the_stage_update_stores(tmp_path, pairs
     # spare: nothing stored, and nothing read where the live threads store
     assert words[3:] == [[0, 8, 0, 8, 8]] * 3
     assert [int(row[1]) for row in got] == [0, 1, 1, 0, 0, 0]
+    assert [int(row[0]) for row in got] == [0] * 6  # none through the read-only path
 
 
 def test_spare_threads_read_no_source_word_that_is_stored():
@@ -82,4 +92,16 @@ def test_spare_threads_read_no_source_word_that_is_stored():
     body = src[a:src.index("\n}\n", a)]
     after = body[body.index("__syncthreads();"):]
     # rows 40..49 (alpha, beta^i, gamma^ij) are only read by this kernel
-    assert re.findall(r"ldA<T, kInt<T>>\(src, P, p, ([^)]*)\)", after) == ["live ? s : 40"]
+    assert re.findall(r"ldA\w*<T, kInt<T>>\(src, P, p, ([^)]*)\)", after) == ["live ? s : 40"]
+
+
+@pytest.mark.parametrize("name,kernel,words", [
+    ("rhs.cu", "k_rhs_quad(const double*", r"\(src, P, p, s\)"),
+    ("rhs.cu", "k_rhs_quad_shared(const double*", r"\(src, P, p, live \? s : 40\)"),
+    ("nest.cu", "k_interface(const double*", r"\(S[AB], \(long long\)f \* P[AB] \+ p[ab]\)"),
+])
+def test_words_that_the_launch_writes_take_ordinary_loads(name, kernel, words):
+    src = _source(name)
+    a = src.index(kernel)
+    reads = re.findall(r"(ld\w*)(?:<T, kInt<T>>)?" + words, src[a:src.index("\n}\n", a)])
+    assert reads and all(r.endswith("_rw") for r in reads), reads
