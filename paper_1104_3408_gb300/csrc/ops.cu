@@ -1369,13 +1369,15 @@ static int launch_batch(const cffyn_shell* sh, const TcBatch& b0, cudaStream_t s
   const int rows = b.W[0].rows;
   // d_r (one class, one row group): the instance with the staged epilogue
   const bool dr = b.nclass == 1 && b.a[0].kind == OP_R && b.W[0].ngroups == 1;
-  const bool persistent = runs_persistent(sh, rows, items, dr);
   const int P = b.a[0].g.P, out_bytes = kTcCols * P * (int)sizeof(double);
-  // d_r's tiles beside the persistent kernel's ring
+  // d_r's tiles beside the persistent kernel's ring: with more than 80 rows there is no
+  // room for them, and lanes that store words a line apart lose more than the kernel
+  // gains, so the one-item kernel, which stages them, keeps these launches (d_r of a
+  // step, us: 90 x 32 x 64 points 111 against 121, 81 x 14 x 28 35 against 42, 96 x 64 x
+  // 128 488 against 492; derivatives of FP64 words there 2096 against 2066)
   const int ring = rows == 48 ? WsCfg<48>::kStage * kRingStages<48, 1> : WsCfg<96>::kStage * kRingStages<96, 1>;
-  const int stage = !dr || (persistent && ring + out_bytes > kTcMaxSmem) ? 0
-                    : persistent && rows == 48 && (P & 1) && P <= kRawRows ? 2
-                                                                           : 1;
+  const bool persistent = runs_persistent(sh, rows, items, dr) && (!dr || ring + out_bytes <= kTcMaxSmem);
+  const int stage = !dr ? 0 : persistent && rows == 48 && (P & 1) && P <= kRawRows ? 2 : 1;
 #define CFFYN_LAUNCH_WS(R_, FI_, ST_)                                                                        \
   k_op_ws<FI_, R_, ST_><<<sh->sm_count, kWsThreads, kRingStages<R_, ST_> * WsCfg<R_>::kStage + ST_ * out_bytes, st>>>( \
       b, exps, pairing, flag)

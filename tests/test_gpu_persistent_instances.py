@@ -1,8 +1,9 @@
 """Every instance of the persistent operator kernel that d_r has: outputs staged as
 one tile beside copied inputs (odd n_r up to 39), staged alone with 48 rows (even
-n_r, 41..47) and with 96, unstaged (n_r > 80).  The shapes are sized from the
-device's SM count and from the lines read off the rule itself, so that a changed
-line keeps them on the persistent side; every one has a ragged last tile.
+n_r, 41..47) and with 96 (up to 80), and the one-item kernel that it has above.
+The shapes are sized from the device's SM count and from the lines read off the rule
+itself, so that a changed line keeps them on the persistent side; every one has a
+ragged last tile.
 
 FP64 words in: the derivatives against the plain FP64 operators, within the bound of
 the 47-bit fixed point (an operator with K columns: 2^-46 (rowsum|W| + K max|W|)

@@ -3,8 +3,8 @@ pipeline wait ends at once): each role leaves its loop by itself, the copies,
 products and bulk stores already issued are waited for, the tensor memory is freed,
 the step reports CFFYN_ETIMEOUT, and with the default bound restored the same
 handle steps as before.  One shape for each form of d_r (inputs copied and outputs
-staged, staged with 48 and with 96 rows, unstaged), large enough that the angular
-derivatives and the filter run persistently too."""
+staged, staged with 48 and with 96 rows, and above 80 rows the one-item kernel),
+large enough that the angular derivatives and the filter run persistently too."""
 
 import pytest
 
