@@ -575,8 +575,11 @@ constexpr int kQPi = 0, kQPh = 10, kQM = 40, kQSlots = 50;
 
 // Warp w takes the sources of d_t Pi_ab with larger index b = w and, w < 3, those
 // of d_t Phi_iab with i = w.
+// Four blocks per SM for a pair state: a step runs it beside the derivative launches,
+// which five blocks of 96 registers hold up (six 9 x 12 x 24 shells stacked, four steps
+// 1917 us, so 1874; alone 16.4 against 15.1 us for 13 x 25 x 50 points).
 template <class T, bool FU>
-__global__ void __launch_bounds__(kRhsBlock)
+__global__ void __launch_bounds__(kRhsBlock, FU ? 4 : 5)
     k_rhs_quad_shared(const double* __restrict__ u, double* __restrict__ src, Geo geo) {
   __shared__ T sm[kQSlots * 32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -673,12 +676,14 @@ __global__ void __launch_bounds__(kRhsBlock)
       }
     }
     const T cPi = -(hal * nnPi);
+    // (a spare thread reads rows that this kernel does not write: its own are being
+    // written by the last point's thread)
+    const double* part_src = live ? src : src + 40 * P;
 #pragma unroll 1
     for (int a = 0; a <= b; ++a) {
       const SymRow ra(a);
       const int s = rb(a);
-      // (a spare thread reads alpha: word s is being written by the last point's own)
-      const T part = ldA_rw<T, kInt<T>>(src, P, p, live ? s : 40);
+      const T part = ldA_rw<T, kInt<T>>(part_src, P, p, s);
       Acc<T> q2;
 #pragma unroll
       for (int c = 0; c < 4; ++c) q2.fma_(-V(kQPi + ra(c)), Piu[c]);

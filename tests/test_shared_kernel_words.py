@@ -92,12 +92,13 @@ def test_spare_threads_read_no_source_word_that_is_stored():
     body = src[a:src.index("\n}\n", a)]
     after = body[body.index("__syncthreads();"):]
     # rows 40..49 (alpha, beta^i, gamma^ij) are only read by this kernel
-    assert re.findall(r"ldA\w*<T, kInt<T>>\(src, P, p, ([^)]*)\)", after) == ["live ? s : 40"]
+    assert re.findall(r"ldA\w*<T, kInt<T>>\((\w+), P, p, ([^)]*)\)", after) == [("part_src", "s")]
+    assert "part_src = live ? src : src + 40 * P;" in after
 
 
 @pytest.mark.parametrize("name,kernel,words", [
     ("rhs.cu", "k_rhs_quad(const double*", r"\(src, P, p, s\)"),
-    ("rhs.cu", "k_rhs_quad_shared(const double*", r"\(src, P, p, live \? s : 40\)"),
+    ("rhs.cu", "k_rhs_quad_shared(const double*", r"\(part_src, P, p, s\)"),
     ("nest.cu", "k_interface(const double*", r"\(S[AB], \(long long\)f \* P[AB] \+ p[ab]\)"),
 ])
 def test_words_that_the_launch_writes_take_ordinary_loads(name, kernel, words):
