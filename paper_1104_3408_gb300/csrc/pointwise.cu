@@ -1016,8 +1016,16 @@ int pw_decompose(const cffyn_shell* sh, const double* in, double* out, bool in_p
 // Whether a point's components are shared out over eight warps: up to one block of
 // 128 points per SM (stages 1-3 / last stage, us, against one thread per tensor
 // group: 8704 points 11 / 18 and 12 / 19, 11250 points 12 / 20 and 14 / 22, 28800 points
-// 27 / 42 and 27 / 36, 67584 points 52 / 79 and 33 / 47).
-static bool recon_shared(const cffyn_shell* sh, unsigned nb) { return nb + sh->beside / 128 <= sh->sm_count; }
+// 27 / 42 and 27 / 36, 67584 points 52 / 79 and 33 / 47).  The component-wise filter's
+// call (copy) has no tensors to share, only values to convert: up to an eighth of
+// that (50 / 54 fields, us for the call, against one thread per group: 882 points
+// 42.6 / 43.4 and 44.9 / 44.8, 2106 points 43.9 / 45.9 and 45.9 / 45.9, 2592 points 46.4 /
+// 49.0 and 46.2 / 47.0, 3744 points 49.4 / 49.0 and 47.5 / 47.2, 8704 points 54.1 / 55.5
+// and 54.1 / 54.1, 10368 points 61.3 / 62.3 and 60.2 / 60.2, 19074 points 69.2 / 73.3 and
+// 69.2 / 69.7).
+static bool recon_shared(const cffyn_shell* sh, unsigned nb, bool copy) {
+  return nb + sh->beside / 128 <= (copy ? sh->sm_count / 8 : sh->sm_count);
+}
 
 // dst (mode 0) is an FP64 array; uf (mixed path): the step's initial state as
 // pairs, read by stages 1-3 and written by the last stage and by mode 0
@@ -1028,8 +1036,9 @@ int pw_reconstruct(const cffyn_shell* sh, const double* sp, double* dst, int mod
   // kernel instance by stage kind: 0 filtered result, 1 stages 1-3, 2 last stage
   const int kind = (mode == 0 || mode == 9) ? 0 : ((mode - 1) % 4 == 3 ? 2 : 1);
   const dim3 gs(blocks_for(g.P, 32), sh->ng ? 2 : 1);
-  const bool shared = recon_shared(sh, grid.x), mixed = sh->d.precision == CFFYN_MIXED;
+  const bool mixed = sh->d.precision == CFFYN_MIXED;
   if (!mixed) uf = nullptr;
+  const bool shared = recon_shared(sh, grid.x, mode == 9 && !uf);
 #define CFFYN_RECON_KIND(T_, K_)                                                                                      \
   (shared ? (void)(k_reconstruct_shared<T_, K_><<<gs, 32 * kShares, 0, st>>>(sp, dst, g, mode, u, U, kacc, uf, dt,    \
                                                                              flag))                                   \
