@@ -44,7 +44,6 @@ void free_tc(TcOp&);
 // pointwise.cu
 int pw_rhs(const cffyn_shell*, const double*, const double*, double*, cudaStream_t);
 int pw_rhs_part(const cffyn_shell*, const double*, const double*, double*, int, bool, bool, cudaStream_t);
-bool pw_rhs_shared(const cffyn_shell*);
 int pw_decompose(const cffyn_shell*, const double*, double*, bool, cudaStream_t);
 int pw_reconstruct(const cffyn_shell*, const double*, double*, int, double*, double*, double*, double*,
                    double, int*, cudaStream_t);

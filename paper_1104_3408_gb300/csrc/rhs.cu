@@ -946,7 +946,6 @@ __global__ void __launch_bounds__(128) k_gauge_rhs(const double* __restrict__ u,
 static bool rhs_shared(const cffyn_shell* sh, unsigned nbr) {
   return 2 * (nbr + sh->beside / kRhsBlock) <= 5ll * sh->sm_count;
 }
-bool pw_rhs_shared(const cffyn_shell* sh) { return rhs_shared(sh, blocks_for((long long)P_all(sh), kRhsBlock)); }
 
 // Shares of the ten symmetric pairs per point in k_rhs_pp: one thread's loop over
 // all ten takes 27 us by itself (its loads wait one after the other), in ten
@@ -961,14 +960,16 @@ static unsigned pp_split(const cffyn_shell* sh, unsigned nb) {
 // stage = 0: all three kernels; 1: sources with Christoffels; 2: quadratic
 // sources; 3: principal parts + boundary.  u_pairs: the state is a pair-stored
 // internal buffer (the stage states of the mixed path); out_pairs: the output
-// is the internal rhs buffer (else an FP64 caller array).
+// is the internal rhs buffer (else an FP64 caller array).  On the mixed path an FP64
+// output goes with an FP64 state where the kernels are shared out and with its pair
+// copy where they are not (pw_rhs): no other combination is instantiated.
 int pw_rhs_part(const cffyn_shell* sh, const double* u, const double* D, double* out, int stage,
                 bool u_pairs, bool out_pairs, cudaStream_t st) {
   Geo g = geo_of(sh);
   const unsigned nb = blocks_for(g.P, 128), nbr = blocks_for(g.P, kRhsBlock), nbs = blocks_for(g.P, 32);
   const bool shared = rhs_shared(sh, nbr);
   const bool mixed = sh->d.precision == CFFYN_MIXED;
-  if (mixed && out_pairs && !u_pairs) {
+  if (mixed && (out_pairs ? !u_pairs : u_pairs == shared)) {
     set_error("internal: right-hand side storage (state %d, output %d) not instantiated", (int)u_pairs,
               (int)out_pairs);
     return CFFYN_EINVAL;
@@ -986,32 +987,33 @@ int pw_rhs_part(const cffyn_shell* sh, const double* u, const double* D, double*
         k_gauge_rhs<ff, false, false><<<nb, 128, 0, st>>>(u, D, sh->H, sh->dH, out, g);
       count_launch();
     }
-#define CFFYN_GAMMA(...)                                                                                       \
-  (shared ? (void)(k_rhs_gamma_shared<__VA_ARGS__><<<nbs, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, \
-                                                                              g, dtH))                         \
-          : (void)(k_rhs_gamma<__VA_ARGS__><<<nbr, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, g, dtH)))
-    if (!mixed)
-      CFFYN_GAMMA(double, false, false);
-    else if (u_pairs && !out_pairs)
-      CFFYN_GAMMA(ff, true, false);
+#define CFFYN_GAMMA(K_, NB_, ...) K_<__VA_ARGS__><<<NB_, kRhsBlock, 0, st>>>(u, sh->H, sh->dH, sh->Rsrc, out, g, dtH)
+    if (!mixed && shared)
+      CFFYN_GAMMA(k_rhs_gamma_shared, nbs, double, false, false);
+    else if (!mixed)
+      CFFYN_GAMMA(k_rhs_gamma, nbr, double, false, false);
+    else if (out_pairs && shared)
+      CFFYN_GAMMA(k_rhs_gamma_shared, nbs, ff, true, true);
+    else if (out_pairs)
+      CFFYN_GAMMA(k_rhs_gamma, nbr, ff, true, true);
     else if (u_pairs)
-      CFFYN_GAMMA(ff, true, true);
+      CFFYN_GAMMA(k_rhs_gamma, nbr, ff, true, false);
     else
-      CFFYN_GAMMA(ff, false, false);
+      CFFYN_GAMMA(k_rhs_gamma_shared, nbs, ff, false, false);
 #undef CFFYN_GAMMA
     count_launch();
   }
   if (stage == 0 || stage == 2) {
-#define CFFYN_QUAD(...)                                                                          \
-  (shared ? (void)(k_rhs_quad_shared<__VA_ARGS__><<<nbs, kRhsBlock, 0, st>>>(u, sh->Rsrc, g))    \
-          : (void)(k_rhs_quad<__VA_ARGS__><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g)))
-    if (!mixed)
-      CFFYN_QUAD(double, false);
-    else if (u_pairs)
-      CFFYN_QUAD(ff, true);
+    if (!mixed && shared)
+      k_rhs_quad_shared<double, false><<<nbs, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
+    else if (!mixed)
+      k_rhs_quad<double, false><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
+    else if (!u_pairs)
+      k_rhs_quad_shared<ff, false><<<nbs, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
+    else if (shared)
+      k_rhs_quad_shared<ff, true><<<nbs, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
     else
-      CFFYN_QUAD(ff, false);
-#undef CFFYN_QUAD
+      k_rhs_quad<ff, true><<<nbr, kRhsBlock, 0, st>>>(u, sh->Rsrc, g);
     count_launch();
   }
   if (stage == 0 || stage == 3) {
@@ -1033,7 +1035,8 @@ int pw_rhs_part(const cffyn_shell* sh, const double* u, const double* D, double*
 // converted once instead of by every kernel that reads it (gamma and quad of
 // 33 x 48 x 96: 142 + 130 us, with the copy 28 + 81 + 91 then, 18.5 + 67 + 66 now).
 int pw_rhs(const cffyn_shell* sh, const double* u, const double* D, double* out, cudaStream_t st) {
-  if (sh->d.precision != CFFYN_MIXED || pw_rhs_shared(sh)) return pw_rhs_part(sh, u, D, out, 0, false, false, st);
+  if (sh->d.precision != CFFYN_MIXED || rhs_shared(sh, blocks_for((long long)P_all(sh), kRhsBlock)))
+    return pw_rhs_part(sh, u, D, out, 0, false, false, st);
   const int rc = pw_to_internal(sh, u, sh->Uf, (long long)sh->nv * (long long)sh->P, st);
   return rc ? rc : pw_rhs_part(sh, sh->Uf, D, out, 0, true, false, st);
 }
