@@ -760,6 +760,8 @@ __device__ __forceinline__ int col_exponent(const TcBatch& B, const OpArgs& a, c
 // thread's 16 words of a line, 8 bytes per load and a line apart across the
 // lanes, were 32 sectors per load: 61 against 56 us for 50 fields of 33 x 48 x 96;
 // odd, so that the lanes' words lie in different banks).
+// 736 threads leave 80 registers each: the instances of pair words spill 116 to 124
+// bytes per thread, 28 to 44 of them read back (<true, 48, 2> none).
 constexpr int kRawRows = 39;
 template <bool FI, int ROWS, int STAGE>
 __global__ void __launch_bounds__(kWsThreads, 1)
@@ -888,11 +890,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         const int words = (int)min((long long)kTcCols, B.a[0].g.ncols - c0) * P;
         const long long* src = reinterpret_cast<const long long*>(B.a[0].in) + c0 * P;
         long long* dst = tile_buf(n);
-        // whole 16 bytes by the bulk copy, the odd last word of the last tile here
-        if (words & 1) dst[words - 1] = __ldg(src + words - 1);
-        const uint32_t bytes = (uint32_t)(words >> 1) * 16;
+        // whole 16 bytes: a sphere has 2 n_theta^2 lines, so columns come in pairs
+        const uint32_t bytes = (uint32_t)words * 8;
         tc::bar_expect_tx(&rawfull[n & 1], bytes);
-        if (bytes) tc::bulk_g2s(dst, src, bytes, &rawfull[n & 1]);
+        tc::bulk_g2s(dst, src, bytes, &rawfull[n & 1]);
       }
       for (int c = n > 2 ? n - 2 : 0; c < n; ++c) tc::bar_wait(&rawfull[c & 1], (c >> 1) & 1, kTcWaitNs);
     }
@@ -1004,7 +1005,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       for (int p0 = h * R; p0 < pend; p0 += CH) {
         uint32_t v[5][CH];
 #pragma unroll
-        for (int d = 0; d < 5; ++d) tc::ld_n(ta + d * ROWS + p0, v[d]);
+        for (int d = 0; d < 5; ++d) tc::ld8(ta + d * ROWS + p0, v[d]);
         tc::ld_wait(v[0]);
 #pragma unroll
         for (int d = 1; d < 5; ++d) tc::tie(v[d]);
@@ -1073,9 +1074,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
   }
 }
 
-// The same products one item per CTA, for launches that do not fill the SMs:
-// their time is one item's latency, which more producer threads with fewer k
-// each shorten.  Producer warps (256 or 512 threads; one column and KQ = 8 or
+// The same products one item per CTA, for launches of few items (runs_persistent:
+// up to one per SM with 96 rows, three with 48, five or more for d_r): their
+// time is mostly one item's latency, which more producer threads with fewer k each
+// shorten, and two CTAs of 48 rows share an SM.  Producer warps (256 or 512 threads; one column and KQ = 8 or
 // 4 consecutive k of every k-step each) slice and, after the last k-step, run
 // the epilogue; one MMA warp copies the operator slices a stage ahead and
 // issues the products.
@@ -1299,7 +1301,7 @@ __global__ void __launch_bounds__(TcCfg<ROWS>::kThreads)
       for (int p0 = g * R; p0 < (g + 1) * R && p0 < prow; p0 += 8) {
         uint32_t v[5][8];
 #pragma unroll
-        for (int d = 0; d < 5; ++d) tc::ld_n(lane + d * ROWS + p0, v[d]);
+        for (int d = 0; d < 5; ++d) tc::ld8(lane + d * ROWS + p0, v[d]);
         tc::ld_wait(v[0]);
 #pragma unroll
         for (int d = 1; d < 5; ++d) tc::tie(v[d]);

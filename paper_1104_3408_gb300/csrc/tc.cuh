@@ -134,21 +134,9 @@ __device__ __forceinline__ void commit(uint64_t* b) {
                : "memory");
 }
 
-// 16 consecutive 32-bit TMEM columns of this thread's lane (warp w reads lanes
+// 8 consecutive 32-bit TMEM columns of this thread's lane (warp w reads lanes
 // 32 (w % 4) .. + 31; taddr carries the lane in bits 16-31).  Not waited on.
-__device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-
-// 8 consecutive 32-bit TMEM columns of this thread's lane.  Not waited on.
-__device__ __forceinline__ void ld_n(uint32_t taddr, uint32_t (&r)[8]) {
+__device__ __forceinline__ void ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                  "=r"(r[7])
@@ -156,40 +144,16 @@ __device__ __forceinline__ void ld_n(uint32_t taddr, uint32_t (&r)[8]) {
                : "memory");
 }
 
-// 4 consecutive 32-bit TMEM columns of this thread's lane.  Not waited on.
-__device__ __forceinline__ void ld_n(uint32_t taddr, uint32_t (&r)[4]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr)
-               : "memory");
-}
-__device__ __forceinline__ void ld_wait(uint32_t (&r)[4]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
-}
-__device__ __forceinline__ void tie(uint32_t (&r)[4]) {
-  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
-}
-
 #define CFFYN_TIE8(r) \
   "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
 
+// Waits for this thread's outstanding TMEM loads.  The registers of r are tied
+// to the wait so that no use of them is scheduled before it.
 __device__ __forceinline__ void ld_wait(uint32_t (&r)[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" : CFFYN_TIE8(r)::"memory");
 }
-__device__ __forceinline__ void tie(uint32_t (&r)[8]) { asm volatile("" : CFFYN_TIE8(r)::"memory"); }
-
-#define CFFYN_TIE16(r)                                                                        \
-  "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), \
-      "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),     \
-      "+r"(r[15])
-
-// Waits for this thread's outstanding TMEM loads.  The registers of r are tied
-// to the wait so that no use of them is scheduled before it.
-__device__ __forceinline__ void ld_wait(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" : CFFYN_TIE16(r)::"memory");
-}
 // Orders the uses of further load destinations after a preceding ld_wait.
-__device__ __forceinline__ void tie(uint32_t (&r)[16]) { asm volatile("" : CFFYN_TIE16(r)::"memory"); }
+__device__ __forceinline__ void tie(uint32_t (&r)[8]) { asm volatile("" : CFFYN_TIE8(r)::"memory"); }
 
 }  // namespace tc
 }  // namespace cffyn
