@@ -1,6 +1,6 @@
 """Per-CTA phase clocks of the tensor-core operator kernel (a diagnostic).
 
-Builds a copy of the library whose k_op_tc sums, for every CTA of the
+Builds a copy of the library whose persistent kernel k_op_ws sums, for every CTA of the
 d_theta + d_phi launch, SM clock64 intervals of each role: the MMA thread's
 waits (operator copies, slices, accumulators) and its issue, a producer warp's
 wait for a free stage, slicing and load issue, an epilogue warp's wait for
@@ -119,6 +119,24 @@ def build():
     return lib
 
 
+def report(buf, shape, mhz):
+    """The table of the clocks read back (a row per CTA: cycles of NAMES, then its
+    items; zero rows: CTAs that recorded nothing)."""
+    import numpy as np
+    rec = buf[buf[:, 12] > 0].astype(np.float64)
+    name = "x".join(str(n) for n in shape)
+    if not len(rec):
+        raise RuntimeError(f"no clocks recorded: the d_theta + d_phi launch of the {name} shell has too few items "
+                           "for the persistent kernel (runs_persistent in csrc/ops.cu)")
+    items = rec[:, 12]
+    lines = [f"d_theta + d_phi launch of the {name} shell: {len(rec)} CTAs, {items.mean():.2f} items each; "
+             f"microseconds at {mhz:.0f} MHz per item (mean, p10, p90)"]
+    for q, nm in enumerate(NAMES):
+        us = rec[:, q] / mhz / (items if q < 11 else 1.0)
+        lines.append(f"{nm:45s} {us.mean():7.2f} {np.percentile(us, 10):7.2f} {np.percentile(us, 90):7.2f}")
+    return "\n".join(lines)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--mhz", type=float, default=2070.0)
@@ -143,14 +161,8 @@ def main():
     buf = np.zeros((1024, 16), dtype=np.uint64)
     if lib.cffyn_instr_read(buf.ctypes.data) != 0:
         raise RuntimeError("reading the phase clocks failed")
-    rec = buf[buf[:, 12] > 0].astype(np.float64)
-    items = rec[:, 12]
-    print(f"d_theta + d_phi launch of the {n_r}x{N}x{J} shell: {len(rec)} CTAs, {items.mean():.2f} items each; "
-          f"microseconds at {args.mhz:.0f} MHz per item (mean, p10, p90)")
-    for q, nm in enumerate(NAMES):
-        us = rec[:, q] / args.mhz / (items if q < 11 else 1.0)
-        print(f"{nm:45s} {us.mean():7.2f} {np.percentile(us, 10):7.2f} {np.percentile(us, 90):7.2f}")
     sh.destroy()
+    print(report(buf, (n_r, N, J), args.mhz))
 
 
 if __name__ == "__main__":
