@@ -606,9 +606,9 @@ static int filter_in_step(cffyn_shell* sh, double* spin, cudaStream_t st, Run&& 
 // read the stage state only) run on the shell's second stream beside the exponent
 // scan and the derivative launches, which they share no buffer with, and join
 // before the principal parts.  Forked at the stage's start: forked after d_r they
-// end after the derivatives (RK4 step, us: 25 x 28 x 56 points 1016 against 881, 33
-// x 48 x 96 2493 against 2408, 49 x 56 x 112 5715 either way; eight shells in a batch
-// 12.85 against 12.23 ms).  Not for the evolved gauge of 54/58 fields
+// end after the derivatives (RK4 step, us: 25 x 28 x 56 points 972 against 879, 33
+// x 48 x 96 2498 against 2414, 49 x 56 x 112 5725 against 5731; eight shells in a batch,
+// two steps, 12.75 against 12.19 ms).  Not for the evolved gauge of 54/58 fields
 // (k_gauge_rhs reads the derivatives) nor under per-group timing.
 template <class Run>
 static int stage_front(cffyn_shell* sh, double* u, int s, cudaStream_t st, Run&& run, bool conc) {

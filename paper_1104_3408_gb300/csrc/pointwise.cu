@@ -577,8 +577,8 @@ __device__ __forceinline__ void reconstruct_update(Scratch<T> sc, const double* 
 // registers and 36 slots, six blocks: 0.423 ms per step on the 33 x 48 x 96
 // shell; eight blocks, 64 registers: 0.340; nine: 0.335, same results).  By now 64
 // us per launch of stages 1-3 (304 MB, 45 us at the copy bandwidth; issue 0.63 per
-// scheduler and cycle, waits for loads and for instructions) and 90 of the last
-// stage.
+// scheduler and cycle, waits for loads and for instructions; 104 bytes of spills)
+// and 90 of the last stage.
 template <class T, bool FD, int KIND>
 __global__ void __launch_bounds__(128, 9) k_reconstruct(const double* __restrict__ sp, double* __restrict__ dst,
                                                      Geo geo, int mode, double* __restrict__ u,
@@ -782,8 +782,8 @@ struct StageUpdate {
 };
 
 // Latency-bound (a few dependent loads and stores per field): 32 warps per SM
-// of at most 64 registers, the state words of the rank-3 legs in flight over
-// their exchange.
+// of at most 64 registers (56 to 68 bytes of spills in the stages), the state words
+// of the rank-3 legs in flight over their exchange.
 template <class T, int KIND>
 __global__ void __launch_bounds__(32 * kShares, 4)
     k_reconstruct_shared(const double* __restrict__ sp, double* __restrict__ dst, Geo geo, int mode, double* __restrict__ u,
@@ -850,11 +850,12 @@ __global__ void __launch_bounds__(32 * kShares, 4)
 
 // Spherical -> Cartesian derivatives: D[3][nf][P] -> out[3][nf][P] (FP64
 // arithmetic; D and out in the given storages).  Setup and API paths only.
-// One thread per point and share of the fields (blockIdx.y, cart_split): the
+// One thread per point and share of the fields (blockIdx.y, cart_grid): the
 // Jacobian is formed once from the tables and applied to every field of the
-// share, whose values are coalesced across the threads.  Bound by the FP64 pipe
-// (eight operations per value at 0.49 T/s: 55 us of the 72 for 50 fields of 33 x 32
-// x 64); with all fields in one thread and the divisions in the kernel 118 us.
+// share, whose values are coalesced across the threads.  Bound by the FP64 pipe:
+// nine operations per value (eight and the zero of z times d_phi) at 0.49 T/s are 62
+// us of the 72 that 50 fields of 33 x 32 x 64 points take; with all fields in one
+// thread and the divisions in the kernel 118 us.
 // status (may be NULL): a status word of the operator launches that produced
 // D; if it is non-zero (a timed-out wait) every output value is a NaN.
 template <bool FI, bool FO>

@@ -938,9 +938,13 @@ __global__ void __launch_bounds__(128) k_gauge_rhs(const double* __restrict__ u,
 // one point per thread per SM.  gamma / quad, us, one thread against four warps per
 // point: 2106 points 14.7 / 13.7 against 8.9 / 7.9, 11250 points 15.5 / 14.0 against
 // 10.5 / 9.8, 28800 points 21.1 / 17.8 against 22.0 / 16.9, 67584 points 32.4 / 31.8
-// against 39.7 / 35.4.  The line lies above where the two meet because the call
-// of an FP64 state goes without its pair copy below it (right-hand side, us: 28800
-// points 132 against 119, 39200 points 167 against 163, 67584 points 216 against 233).
+// against 39.7 / 35.4 (quad by now, at four blocks per SM, 15.1 for 16250 points, 28.6
+// for 39200).  The line lies above where the two meet because the call of an FP64
+// state goes without its pair copy below it (right-hand side, us: 28800 points 132
+// against 119, 39200 points 167 against 163, 67584 points 216 against 233).  The
+// kernels of a step run beside its derivative launches, where the same line holds:
+// at 1.5 blocks per SM instead, RK4 step, us: 31250 points 799 against 775, 35280 points
+// 791 against 777, 39200 points 883 against 879, 44064 points 978 against 984.
 // Blocks of a batch's other classes count too: beside them the shorter chain buys
 // nothing and the repeated work costs (batch of eight shells 14.7 against 15.4 ms).
 static bool rhs_shared(const cffyn_shell* sh, unsigned nbr) {
