@@ -172,7 +172,8 @@ def _time_steps(sh, u, dt, K, flush, torch, use_async=True):
     return total
 
 
-# Kernel families of the step and the trace phases each one runs in.
+# Kernel families of the step and the trace phases each one runs in (k_op_tc:
+# the operator launches, k_op_ws where they are persistent).
 FAMILIES = {
     "k_op_tc": ["d_r", "d_theta_phi", "dft_fwd", "project", "dft_inv"],
     "k_reconstruct": ["reconstruct"],
@@ -224,7 +225,7 @@ def _pointwise_bytes(w, phase):
 
 
 def _op_sources_sha():
-    """sha256 of the sources that define the operator kernel k_op_tc."""
+    """sha256 of the sources that define the operator kernels k_op_ws and k_op_tc."""
     import hashlib
     h = hashlib.sha256()
     for name in ("ops.cu", "tc.cuh", "common.cuh"):
@@ -240,7 +241,7 @@ def _op_traffic(w):
     import re
     path = os.path.join(ROOT, "profiles", f"k_op_tc_dram_{w['name']}.md")
     if not os.path.exists(path):
-        return None, "no single-kernel DRAM capture of k_op_tc for this workload"
+        return None, "no single-kernel DRAM capture of the operator kernels for this workload"
     with open(path) as fh:
         text = fh.read()
     sha = re.search(r"sources_sha256:\s*([0-9a-f]{64})", text)
@@ -248,7 +249,7 @@ def _op_traffic(w):
     if not sha or not val:
         return None, "capture summary without sources_sha256 / dram_bytes_per_step"
     if sha.group(1) != _op_sources_sha():
-        return None, "capture taken on other k_op_tc sources (stale)"
+        return None, "capture taken on other operator kernel sources (stale)"
     return float(val.group(1)), f"profiles/k_op_tc_dram_{w['name']}.md"
 
 
@@ -303,10 +304,10 @@ def _roofline(w, per_step, launches, hbm, bf16s, peak_kind):
                               "method_tflops": 4 * _op_flops(w, ph) / tl / 1e12,
                               "tensor_pipe_frac": PAIRS[ph] * 4 * _op_flops(w, ph) / tl / 1e12 / bf16s}
         traffic, tsrc = _op_traffic(w)
-        return {"bound": "tensor", "kernel": "k_op_tc (all operator launches of the step)",
+        return {"bound": "tensor", "kernel": "k_op_ws / k_op_tc (all operator launches of the step)",
                 "achieved": achieved, "peak": bf16s, "unit": "TFLOP/s", "frac": achieved / bf16s,
                 "traffic": traffic, "traffic_source": tsrc,
-                "traffic_scope": "DRAM bytes per step, all k_op_tc launches",
+                "traffic_scope": "DRAM bytes per step, all operator launches",
                 "peak_source": f"bf16_tflops_sustained ({peak_kind})",
                 "work": "the method's FP64 operator flops, 2n_r + 16N + 2(L+1) per pt-field per substep "
                         "(no emulation overhead)",
@@ -687,7 +688,7 @@ def run_batch(args, rank, local_rank, ws, dist):
         fl += 4.0 * (deriv + filt) * _shell_units(d)
         issued += 4.0 * (26 * deriv + 21 * filt) * _shell_units(d)
     achieved = fl * args.steps / (t_ms * 1e-3) / 1e12
-    roof = {"bound": "tensor", "kernel": "k_op_tc (operator work over the whole batch step time)",
+    roof = {"bound": "tensor", "kernel": "k_op_ws / k_op_tc (operator work over the whole batch step time)",
             "achieved": achieved, "peak": bf16s, "unit": "TFLOP/s", "frac": achieved / bf16s,
             "traffic": None, "traffic_source": "no single-kernel capture of the batch",
             "peak_source": f"bf16_tflops_sustained ({peak_kind})",
@@ -897,7 +898,7 @@ def run_derivs_sweep(args):
         del outs, u
         torch.cuda.empty_cache()
     return {"mode": "derivs_sweep", "fields": nv, "method_note":
-            "matrix_mixed: split-precision BF16 digit products on tcgen05 (k_op_tc); matrix_fp64: "
+            "matrix_mixed: split-precision BF16 digit products on tcgen05 (k_op_ws / k_op_tc); matrix_fp64: "
             "FP64 matrices (k_op_fp64); fft_fp64: cuFFT D2Z/Z2D with the library's own extension, "
             "recurrence and transpose kernels; all followed by the same chain-rule kernel",
             "timing": "median of 5 calls after 2 warm-ups, CUDA events, L2 flushed before each call",
