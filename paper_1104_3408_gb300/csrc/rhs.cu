@@ -575,11 +575,12 @@ constexpr int kQPi = 0, kQPh = 10, kQM = 40, kQSlots = 50;
 
 // Warp w takes the sources of d_t Pi_ab with larger index b = w and, w < 3, those
 // of d_t Phi_iab with i = w.
-// Four blocks per SM for a pair state: a step runs it beside the derivative launches,
-// which five blocks of 96 registers hold up (six 9 x 12 x 24 shells stacked, four steps
-// 1917 us, so 1874; alone 16.4 against 15.1 us for 13 x 25 x 50 points).
+// 112 registers, four blocks per SM, for a pair state: a step runs it beside the
+// derivative launches, which five blocks of 96 registers hold up (six 9 x 12 x 24
+// shells stacked, four steps 1917 us, so 1874), and with 127 the step takes longer too
+// (two steps of 25 x 24 x 48 points 1358 us, so 1346).
 template <class T, bool FU>
-__global__ void __launch_bounds__(kRhsBlock, FU ? 4 : 5)
+__global__ void __launch_bounds__(kRhsBlock) __maxnreg__(FU ? 112 : 96)
     k_rhs_quad_shared(const double* __restrict__ u, double* __restrict__ src, Geo geo) {
   __shared__ T sm[kQSlots * 32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
